@@ -5,10 +5,9 @@
 //   S_R(y) = U_i(y) U_i(y+i) ... U_i(y+(R-1)i),  T_T(y) = U_t(y) ... U_t(y+(T-1)t),
 //   A = S_R(x) T_T(x+Ri),  B = T_T(x) S_R(x+Tt),  loop = (1/2) Tr A B^dag = A . B,
 // line products left to right, binary32 per loop (the link-arithmetic
-// contract), binary64 mean over x and i = 0, 1, 2.  One launch per T: each
-// thread takes (site, direction) items and, for R = 1 .. rmax, extends S_R
-// and the line at height T by one link and walks T_T(x+Ri); per-R sums in
-// registers, block partials in a fixed order, so the result is reproducible.
+// contract); the mean over x and i = 0, 1, 2 is exact to 2^-44 per loop in
+// fixed point (wilson_tile_kernel), or binary64 for configurations whose loops
+// leave the fixed-point range (wilson_kernel).
 #include <algorithm>
 
 #include "observables.cuh"
@@ -21,6 +20,277 @@ constexpr int kWilsonThreads = 256;
 constexpr int kWilsonMaxR = 16;
 constexpr int kWilsonMaxT = 64;
 
+// ------------------------------------------------------- tiled kernel
+// All loops of an (i, t) plane stay inside the plane, so a block takes a tile
+// of bx x bt sites of one plane (one site per thread) and a chunk of up to
+// 8 x 8 extents (R, T) and works from shared memory:
+//   * the lines S_R of the rows the tile's tops reach, for every R of the
+//     chunk, are formed once (s_buf);
+//   * T_T is extended by one link per step of T and published with the
+//     columns x + R next to the tile (tt_buf, double buffered: one block
+//     barrier per step);
+//   * a loop is then two shared-memory loads, the products A and B and their
+//     scalar product: 36 of its about 50 instructions.
+// The walk it replaces formed T_T(x + Ri) again for every R and T from global
+// loads (T + 2 loads and T + 2 products per loop), and added every loop in
+// binary64, of which this chip starts two per clock and SM.  Here the loop
+// value x is split exactly into integers, x = h 2^-21 + l 2^-43 (l rounded to
+// nearest), by adding and subtracting 6 = 1.5 2^2, whose binary32 neighbours
+// lie 2^-21 apart; the warp adds h and l with integer reductions, the block
+// and the grid with integer atomics, so the sum does not depend on any order
+// and is within 2^-44 per loop of the exact one.  |x| < 2 is required (unit
+// links give |x| <= 1); a loop outside (links that are not unit, NaN) sets
+// *flag, and the host then takes the binary64 path.
+// Bound: instruction issue (71% of the slots; 82 warp instructions per 32
+// loops, the tile's preparation included).  24^4, all loops up to 8 x 8: 1243
+// -> 219 us per call, of it 189 us (ncu) in this kernel.
+constexpr int kLoopChunk = 8;          // extents R and T per block
+constexpr int kTileThreads = 256;      // most sites of a tile
+constexpr int kTileMaxBx = 64;         // most columns of a tile
+constexpr float kSplit = 6.0f;         // its neighbours lie 2^-21 apart
+constexpr unsigned int kSplitBits = 0x40C00000u;
+constexpr int kTopPitch = kLoopChunk + 1;  // float4 per site of s_buf: an odd pitch keeps 16-byte reads conflict-free
+
+struct LoopTiles {
+    int bx, bt;          // tile extents along i and t
+    int nx, nt, nr, ntc;  // tiles along i, along t, chunks of R, chunks of T
+};
+
+__device__ __forceinline__ int wrap_once(int c, int extent) { return c >= extent ? c - extent : c; }
+
+// Shared memory of a tile with extents bx x bt, in float4: [0] the two T_T
+// buffers, which first hold the staged U_i (rows t0 + tc0 .. + bt + 8, columns
+// x0 .. x0 + ucols - 1, all of them when they cover the extent), [1] the staged
+// U_t (rows t0 + tc0 .. + bt + 7), [2] s_buf.
+struct TileSmem {
+    int ucols, ut, s, total;
+};
+
+__host__ __device__ inline TileSmem tile_smem(int bx, int bt, int ns, int r0)
+{
+    TileSmem m;
+    m.ucols = bx + r0 + kLoopChunk < ns ? bx + r0 + kLoopChunk : ns;
+    const int buf = 2 * bt * (bx + kLoopChunk), ui = (bt + kLoopChunk) * m.ucols;
+    m.ut = buf > ui ? buf : ui;
+    m.s = m.ut + (bt + kLoopChunk - 1) * m.ucols;
+    m.total = m.s + kTopPitch * (bt + kLoopChunk) * bx;
+    return m;
+}
+
+// FULL: the chunk has all eight R (no test per R in the inner loop).
+template <bool FULL>
+__global__ void __launch_bounds__(kTileThreads, 3)
+    wilson_tile_kernel(const float4 *__restrict__ L, Geom g, LoopTiles tl, int rmax, int tmax,
+                       unsigned long long *__restrict__ slots, int nslots, unsigned int *__restrict__ flag)
+{
+    extern __shared__ float4 sm[];
+    // [T][R][h, l] of the chunk, modulo 2^32; starts at minus what the bits of
+    // 6 add up to over the block's warps
+    __shared__ unsigned int s_sum[2 * kLoopChunk * kLoopChunk];
+    const int pitch = tl.bx + kLoopChunk;  // a T_T row: the tile's columns, then x + R
+    const int buf_len = tl.bt * pitch;
+    uint32_t b = blockIdx.x;
+    const int r0 = (int)(b % (uint32_t)tl.nr) * kLoopChunk;
+    b /= (uint32_t)tl.nr;
+    const int tc0 = (int)(b % (uint32_t)tl.ntc) * kLoopChunk;
+    b /= (uint32_t)tl.ntc;
+    // the plane: direction i and the two transverse coordinates, the first
+    // fastest (planes of neighbouring blocks share 32-byte sectors)
+    const int q0 = (int)(b % (uint32_t)g.ns);
+    b /= (uint32_t)g.ns;
+    const int q1 = (int)(b % (uint32_t)g.ns);
+    b /= (uint32_t)g.ns;
+    const int x0 = (int)(b % (uint32_t)tl.nx) * tl.bx;
+    b /= (uint32_t)tl.nx;
+    const int t0 = (int)(b % (uint32_t)tl.nt) * tl.bt;
+    const int i = (int)(b / (uint32_t)tl.nt);
+    const int rcnt = FULL ? kLoopChunk : min(kLoopChunk, rmax - r0), tcnt = min(kLoopChunk, tmax - tc0);
+    const TileSmem lay = tile_smem(tl.bx, tl.bt, g.ns, r0);
+    float4 *const s_ui = sm, *const s_ut = sm + lay.ut;
+    float4 *const s_buf = sm + lay.s;  // [row t0 + tc0 + j][column][R]
+    const int stride_i = g.stride[i];
+    const int lex_plane = q0 * g.stride[i == 0 ? 1 : 0] + q1 * g.stride[i == 2 ? 1 : 2];
+    const float4 *const Li = L + link_index(g, i, 0, 0);
+    const float4 *const Lt = L + link_index(g, 3, 0, 0);
+    auto link = [&](const float4 *dir, int a, int t) {  // 0 <= a < ns, 0 <= t < nt
+        const int lex = t * g.vs + a * stride_i + lex_plane;
+        const int parity = (a + t + q0 + q1) & 1;
+        return __ldg(dir + (uint32_t)parity * (uint32_t)g.vh + (uint32_t)(lex >> 1));
+    };
+
+    for (int q = threadIdx.x; q < 2 * kLoopChunk * kLoopChunk; q += blockDim.x)
+        s_sum[q] = 0u - blockDim.x * kSplitBits;
+    for (int q = threadIdx.x; q < (tl.bt + tcnt) * lay.ucols; q += blockDim.x) {
+        const int j = q / lay.ucols, d = q - j * lay.ucols;
+        const int a = (x0 + d) % g.ns, t = (t0 + tc0 + j) % g.nt;
+        s_ui[q] = link(Li, a, t);
+        if (j < tl.bt + tcnt - 1) s_ut[q] = link(Lt, a, t);
+    }
+    __syncthreads();
+    // S_R on the rows t0 + tc0 + j; d: the column's place in the staged row,
+    // which wraps only when the row holds the whole extent
+    for (int q = threadIdx.x; q < (tl.bt + tcnt) * tl.bx; q += blockDim.x) {
+        const int j = q / tl.bx;
+        const float4 *const u = s_ui + j * lay.ucols;
+        float4 *const to = s_buf + q * kTopPitch;
+        int d = q - j * tl.bx;
+        float4 s = u[d];
+        if (r0 == 0) to[0] = s;
+        for (int r = 1; r < r0 + rcnt; ++r) {
+            d = wrap_once(d + 1, lay.ucols);
+            s = qmul(s, u[d]);
+            if (r >= r0) to[r - r0] = s;
+        }
+    }
+    // this thread's site: column c, row k of the tile; threads past the tile
+    // and sites past the plane's edge compute on clamped indices and add zero
+    // (their s_bot is zero)
+    const int site = min((int)threadIdx.x, tl.bx * tl.bt - 1);
+    const int k = site / tl.bx, c = site - k * tl.bx;
+    const bool active = (int)threadIdx.x < tl.bx * tl.bt && x0 + c < g.ns && t0 + k < g.nt;
+    // the column next to the tile that this thread extends: h < rcnt <= bx
+    const int hk = (int)threadIdx.x / rcnt, h = (int)threadIdx.x - hk * rcnt;
+    const bool halo = hk < tl.bt;
+    // T_T at the site, at its column + r0, and at the halo column, after the
+    // steps before this chunk (walked from global memory; none in the first)
+    float4 tt0 = make_float4(1.0f, 0.0f, 0.0f, 0.0f), tb = tt0, th = tt0;
+    float4 s_bot[kLoopChunk];
+    __syncthreads();  // s_buf is complete, the staged U_i is done with
+    if (tc0 == 0) {
+#pragma unroll
+        for (int r = 0; r < kLoopChunk; ++r) s_bot[r] = s_buf[site * kTopPitch + min(r, rcnt - 1)];
+    } else {  // the site's own row is not among the staged ones
+        int a = (x0 + c) % g.ns;
+        const int t = (t0 + k) % g.nt;
+        float4 s = link(Li, a, t);
+        for (int r = 1; r <= r0; ++r) {
+            a = wrap_once(a + 1, g.ns);
+            s = qmul(s, link(Li, a, t));
+        }
+        s_bot[0] = s;
+#pragma unroll
+        for (int r = 1; r < kLoopChunk; ++r) {
+            a = wrap_once(a + 1, g.ns);
+            if (r < rcnt) s = qmul(s, link(Li, a, t));
+            s_bot[r] = s;
+        }
+        auto walk = [&](int col, int row) {
+            const int ca = col % g.ns;
+            int ct = row % g.nt;
+            float4 p = link(Lt, ca, ct);
+            for (int step = 1; step < tc0; ++step) {
+                ct = wrap_once(ct + 1, g.nt);
+                p = qmul(p, link(Lt, ca, ct));
+            }
+            return p;
+        };
+        tt0 = walk(x0 + c, t0 + k);
+        if (r0 > 0) tb = walk(x0 + c + r0, t0 + k);
+        if (halo) th = walk(x0 + r0 + tl.bx + h, t0 + hk);
+    }
+    if (!active) {
+#pragma unroll
+        for (int r = 0; r < kLoopChunk; ++r) s_bot[r] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+    const float4 *ut = s_ut + k * lay.ucols + c;
+    const int tb_off = wrap_once(c + r0, lay.ucols) - c;
+    const float4 *ut_h = s_ut + hk * lay.ucols + wrap_once(tl.bx + r0 + h, lay.ucols);
+    float4 *own_to = sm + k * pitch + c, *halo_to = sm + hk * pitch + tl.bx + h;
+    const float4 *top = s_buf + (site + tl.bx) * kTopPitch;  // the site one step of T above, then two ...
+
+    const int lane = threadIdx.x & 31;
+    bool outside = false;
+    unsigned int acc_h = 0, acc_l = 0;  // lane (T & 3) 8 + R of the current four steps of T
+    auto flush = [&](int tt_first) {
+        const int idx = 2 * (tt_first * kLoopChunk + lane);
+        atomicAdd(&s_sum[idx], acc_h);
+        atomicAdd(&s_sum[idx + 1], acc_l);
+        acc_h = acc_l = 0;
+    };
+    for (int tt = 0; tt < tcnt; ++tt) {
+        const int flip = (tt & 1) * buf_len;
+        const bool first = tc0 + tt == 0;  // block-uniform
+        const float4 u = *ut;
+        tt0 = first ? u : qmul(tt0, u);
+        if (r0 > 0) {
+            const float4 ub = ut[tb_off];
+            tb = first ? ub : qmul(tb, ub);
+        } else {
+            tb = tt0;
+        }
+        if ((int)threadIdx.x < tl.bx * tl.bt) own_to[flip] = tb;
+        if (halo) {
+            const float4 uh = *ut_h;
+            th = first ? uh : qmul(th, uh);
+            halo_to[flip] = th;
+        }
+        ut += lay.ucols;
+        ut_h += lay.ucols;
+        __syncthreads();
+        const float4 *const row = own_to + flip + 1;
+        const int acc_r = lane - (tt & 3) * kLoopChunk;  // the R whose sums this lane takes
+#pragma unroll
+        for (int r = 0; r < kLoopChunk; ++r) {
+            if (r < rcnt) {  // block-uniform
+                const float4 A = qmul(s_bot[r], row[r]);
+                const float4 B = qmul(tt0, top[r]);
+                const float x = chain4(A.x, B.x, A.y, B.y, A.z, B.z, A.w, B.w);
+                outside |= !(fabsf(x) < 2.0f);
+                const float y = __fadd_rn(x, kSplit);
+                const float z = __fmaf_rn(__fsub_rn(x, __fsub_rn(y, kSplit)), 0x1p22f, kSplit);
+                const unsigned int hs = __reduce_add_sync(0xffffffffu, __float_as_uint(y));
+                const unsigned int ls = __reduce_add_sync(0xffffffffu, __float_as_uint(z));
+                if (acc_r == r) {
+                    acc_h += hs;
+                    acc_l += ls;
+                }
+            }
+        }
+        top += tl.bx * kTopPitch;
+        if ((tt & 3) == 3) flush(tt - 3);
+    }
+    if (tcnt & 3) flush(tcnt & ~3);
+    if (__any_sync(0xffffffffu, outside) && lane == 0) atomicOr(flag, 1u);
+    __syncthreads();
+    // the block's sums into its slot: [slot][R][T][h, l]
+    unsigned long long *const slot = slots + (size_t)(blockIdx.x % (uint32_t)nslots) * (size_t)(2 * rmax * tmax);
+    for (int q = threadIdx.x; q < kLoopChunk * tcnt; q += blockDim.x) {
+        const int r = q & (kLoopChunk - 1), tt = q >> 3;
+        if (r >= rcnt) continue;
+        unsigned long long *const d = slot + 2 * ((r0 + r) * tmax + tc0 + tt);
+        const int vh = (int)s_sum[2 * q], vl = (int)s_sum[2 * q + 1];
+        if (vh) atomicAdd(d, (unsigned long long)(long long)vh);
+        if (vl) atomicAdd(d + 1, (unsigned long long)(long long)vl);
+    }
+}
+
+// out[o] = scale (sum over slots), one warp per output; out[n_out] = the flag.
+__global__ void wilson_tile_finish_kernel(const unsigned long long *__restrict__ slots, int nslots, int n_out,
+                                          double scale, const unsigned int *__restrict__ flag,
+                                          double *__restrict__ out)
+{
+    const int o = blockIdx.x;
+    long long h = 0, l = 0;
+    for (int s = threadIdx.x; s < nslots; s += 32) {
+        h += (long long)slots[((size_t)s * n_out + o) * 2];
+        l += (long long)slots[((size_t)s * n_out + o) * 2 + 1];
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+        h += __shfl_down_sync(0xffffffffu, h, off);
+        l += __shfl_down_sync(0xffffffffu, l, off);
+    }
+    if (threadIdx.x == 0) {
+        out[o] = ((double)h * 0x1p-21 + (double)l * 0x1p-43) * scale;
+        if (o == 0) out[n_out] = *flag ? 1.0 : 0.0;
+    }
+}
+
+// ------------------------------------------------------ binary64 kernel
+// One launch per T: each thread takes (site, direction) items and, for R = 1
+// .. rmax, extends S_R and the line at height T by one link and walks
+// T_T(x+Ri); per-R binary64 sums in registers, block partials in a fixed
+// order.  Takes any links, so it finishes the calls whose loops the tiled
+// kernel's fixed point does not hold (24^4 up to 8 x 8: 1.2 ms).
 struct Site {
     int c[4];
 };
@@ -128,6 +398,50 @@ static cudaError_t launch_wilson(su2_lattice *lat, int rmax, int tmax, double *d
     return cudaGetLastError();
 }
 
+// Enqueues the tiled kernel: tiles of whole rows (up to 64 columns) and as
+// many time slices as fit 256 threads.  The sums live in the reduction
+// scratch, in as many slots as fit (blocks spread over the slots, so their
+// atomics meet rarely), the results behind them: rmax tmax values and the
+// flag.  *d_out: their device address.
+static cudaError_t launch_tiles(su2_lattice *lat, int rmax, int tmax, double **d_out)
+{
+    const Geom g = geom_of(lat);
+    const int n_out = rmax * tmax;
+    LoopTiles tl;
+    tl.bx = std::min(g.ns, kTileMaxBx);
+    tl.bt = std::min(lat->nt, std::max(1, kTileThreads / tl.bx));
+    tl.nx = (g.ns + tl.bx - 1) / tl.bx;
+    tl.nt = (lat->nt + tl.bt - 1) / tl.bt;
+    tl.bt = (lat->nt + tl.nt - 1) / tl.nt;  // even tiles
+    tl.nr = (rmax + kLoopChunk - 1) / kLoopChunk;
+    tl.ntc = (tmax + kLoopChunk - 1) / kLoopChunk;
+    const int nslots = std::min(256, (lat->scratch.partials_cap - n_out - 2) / (2 * n_out));
+    unsigned long long *slots = (unsigned long long *)lat->scratch.partials;
+    unsigned int *flag = (unsigned int *)(slots + (size_t)nslots * 2 * n_out);
+    *d_out = (double *)(flag + 2);
+    cudaError_t e = cudaMemsetAsync(slots, 0, sizeof(double) * ((size_t)nslots * 2 * n_out + 1), lat->stream);
+    if (e != cudaSuccess) return e;
+    const size_t smem = sizeof(float4) * (size_t)tile_smem(tl.bx, tl.bt, g.ns, (tl.nr - 1) * kLoopChunk).total;
+    const auto kernel = rmax % kLoopChunk == 0 ? wilson_tile_kernel<true> : wilson_tile_kernel<false>;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const unsigned int blocks = 3u * (unsigned int)(g.ns * g.ns) * (unsigned int)(tl.nx * tl.nt * tl.nr * tl.ntc);
+    const int threads = std::max(32, (tl.bx * tl.bt + 31) & ~31);
+    kernel<<<blocks, threads, smem, lat->stream>>>(lat->links, g, tl, rmax, tmax, slots, nslots, flag);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    wilson_tile_finish_kernel<<<n_out, 32, 0, lat->stream>>>(slots, nslots, n_out, 1.0 / (6.0 * (double)g.vh), flag,
+                                                             *d_out);
+    return cudaGetLastError();
+}
+
+// The binary64 path: d_out holds rmax tmax values.
+static cudaError_t launch_walks(su2_lattice *lat, int rmax, int tmax, double *d_out)
+{
+    return rmax <= 4   ? launch_wilson<4>(lat, rmax, tmax, d_out)
+           : rmax <= 8 ? launch_wilson<8>(lat, rmax, tmax, d_out)
+                       : launch_wilson<16>(lat, rmax, tmax, d_out);
+}
+
 }  // namespace su2
 
 using namespace su2;
@@ -140,15 +454,24 @@ extern "C" su2_status su2_wilson_loops(su2_lattice *lat, int rmax, int tmax, dou
         return SU2_E_INVAL;
     }
     DeviceGuard guard(lat->device);
-    const size_t bytes = sizeof(double) * (size_t)rmax * (size_t)tmax;
+    const size_t n_out = (size_t)rmax * (size_t)tmax;
+    const size_t bytes = sizeof(double) * n_out;
+    double host[kWilsonMaxR * kWilsonMaxT + 1];
+    double *d_tiles = nullptr;
+    SU2_CUDA(launch_tiles(lat, rmax, tmax, &d_tiles));
+    SU2_CUDA(cudaMemcpyAsync(host, d_tiles, bytes + sizeof(double), cudaMemcpyDeviceToHost, lat->stream));
+    SU2_CUDA(cudaStreamSynchronize(lat->stream));
+    if (host[n_out] == 0.0) {
+        std::copy(host, host + n_out, out);
+        return SU2_OK;
+    }
+    // a loop outside (-2, 2)
     double *d_out = (double *)device_alloc(bytes, lat->device, lat->stream);
     if (!d_out) {
         set_last_error("device allocation for the Wilson loops failed");
         return SU2_E_NOMEM;
     }
-    cudaError_t e = rmax <= 4 ? launch_wilson<4>(lat, rmax, tmax, d_out)
-                   : rmax <= 8 ? launch_wilson<8>(lat, rmax, tmax, d_out)
-                               : launch_wilson<16>(lat, rmax, tmax, d_out);
+    cudaError_t e = launch_walks(lat, rmax, tmax, d_out);
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, d_out, bytes, cudaMemcpyDeviceToHost, lat->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(lat->stream);
     device_free(d_out, bytes, lat->device, lat->stream);
