@@ -5,6 +5,7 @@
 // memory), and an Adam update.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstring>
 #include <vector>
@@ -111,44 +112,137 @@ extern "C" su2_status su2_selftest_mma(const uint16_t *A, const uint16_t *B, int
 
 // ============================================================== training
 #include "learned.cuh"
+#include "observables.cuh"
 
 namespace su2 {
 namespace train {
 
-constexpr int kRows = 128;      // samples per CTA (the MMA M dimension)
-constexpr int kPad = 33;        // row stride of the fp32 stashes (bank-conflict free)
+// A step works on 128 samples per CTA (the MMA M dimension) with four threads
+// per sample: thread (row, part) holds columns 8 part .. 8 part + 7 of the
+// sample's 32-wide rows, the split in which tensor memory hands the
+// accumulator to four warps per 32 rows, and in which the network's outputs
+// fall apart (bin widths, bin heights, knot derivatives 0..7, derivative 8),
+// so the softmax and softplus work of a sample runs on four warps at once.
+// The gradient sums over the 128 rows (rows in order, binary32) take all 16
+// warps, four outputs per thread: one 16-byte broadcast and one conflict-free
+// load per four multiply-adds.  Batches of 4096 fill 32 SMs with one CTA each,
+// so a step is latency, not throughput: TRAIN_FIGURES
+constexpr int kRows = 128;                   // samples per CTA
+constexpr int kParts = 4;                    // threads per sample
+constexpr int kTrainThreads = kRows * kParts;
+constexpr int kPitch = 36;                   // row pitch of the binary32 stashes: 16-byte rows, conflict-free columns
 constexpr int kGradSlots = learned::kTrainable + 1;  // 1945 gradients + loss sum
 
-// -log q(a | o) = log 2 + log f'(f^{-1}(a)) for the spline of outputs o, and
-// its gradient with respect to o: implicit differentiation of f(z) = a at
-// fixed a through the bin's knots, then the knot sums, the softmax and the
-// softplus (binary32; the same formulas as the binary64 reference).
-__device__ float nll_and_grad(const float (&o)[learned::kOut], float a, float (&g)[learned::kOut])
+struct StepParams {
+    const float *w;            // 1947 master weights (fp32)
+    const float2 *pairs;       // (beta k, a0)
+    long long n_pairs;
+    int explicit_rows;         // 1: row r of CTA b is pair b*128 + r; 0: random pairs
+    uint32_t step, k0, k1;     // Philox key and counter for random pairs
+    float *partials;           // [gridDim.x][kGradSlots]
+    unsigned int *err;
+};
+
+__device__ __forceinline__ uint32_t to_bf16(float f)
+{
+    const uint32_t u = __float_as_uint(f);
+    return (u + 0x7FFFu + ((u >> 16) & 1u)) >> 16;
+}
+
+struct Smem {
+    unsigned char A[kRows * 32 * 2];     // activation tile (A operand)
+    unsigned char W2[32 * 32 * 2];       // B: W2 (n = output j, k = input i)
+    unsigned char W3[32 * 32 * 2];       // B: W3 (n = output o, padded to 32)
+    unsigned char W3T[32 * 32 * 2];      // B: W3^T (n = j, k = o padded)
+    unsigned char W2T[32 * 32 * 2];      // B: W2^T (n = i, k = j)
+    float h1[kRows][kPitch], h2[kRows][kPitch], go[kRows][kPitch], dz2[kRows][kPitch], dz1[kRows][kPitch];
+    float w1[32], b1[32], b2[32], b3[32];
+    float knot[2][learned::kBins + 1][kRows];  // x_0 .. x_8, y_0 .. y_8 of each sample
+    float der[learned::kBins + 1][kRows];
+    float g_knot[2][2][kRows];           // gradient at knots k, k + 1 of x and y
+    float g_der[2][kRows];               // gradient at derivatives k, k + 1
+    int bin[kRows];
+    float s_in[kRows];
+    float loss[kRows];
+    uint64_t mbar;
+    uint32_t tmem_base;
+};
+
+// Dependent launches (the step and the Adam kernel alternate): let the next
+// grid of the stream start its independent prologue, and wait until the
+// previous grid has finished and its writes are visible.
+__device__ __forceinline__ void release_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// One MMA pass: D (tmem) = A (smem tile, 128 x 32) * B^T (32 x 32), then this
+// thread's eight columns of its row of D into v.  Every thread must call it
+// (barriers inside).
+__device__ bool mma_pass(Smem &sm, const unsigned char *B, uint32_t taddr, uint32_t &phase, float (&v)[8])
+{
+    tc::fence_smem_to_async();
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    if (threadIdx.x == 0) {
+        const uint32_t idesc = tc::idesc_bf16_f32(128, 32);
+        for (int j = 0; j < 2; ++j) {
+            const uint64_t ad = tc::smem_desc(tc::smem_addr(sm.A) + 256u * j, 128u, 512u);
+            const uint64_t bd = tc::smem_desc(tc::smem_addr(B) + 256u * j, 128u, 512u);
+            tc::mma_bf16(taddr, ad, bd, idesc, j > 0 ? 1u : 0u);
+        }
+        tc::mma_commit(&sm.mbar);
+    }
+    bool ok = tc::mbar_wait(&sm.mbar, phase, kMbarPolls);
+    if (!ok) ok = tc::mbar_wait(&sm.mbar, phase, kMbarPolls);
+    phase ^= 1u;
+    tc::fence_after_sync();
+    // a warp reads the 32 lanes of its place in its group of four
+    const uint32_t warp = threadIdx.x >> 5;
+    if (ok) {
+        tc::tmem_load8(taddr + ((warp & 3u) * 32u << 16) + (warp >> 2) * 8u, v);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = 0.0f;
+    }
+    tc::fence_before_sync();
+    __syncthreads();  // every thread has read D and A before either is overwritten
+    return ok;
+}
+
+// This thread's eight columns: binary32 into the stash, BF16 into the A tile
+// (one row of one core matrix).
+__device__ __forceinline__ void stash_row(float (&stash)[kRows][kPitch], int row, int part, const float (&v)[8])
+{
+    float4 *const to = (float4 *)&stash[row][8 * part];
+    to[0] = make_float4(v[0], v[1], v[2], v[3]);
+    to[1] = make_float4(v[4], v[5], v[6], v[7]);
+}
+
+__device__ __forceinline__ void put_row_bf16(Smem &sm, int row, int part, const float (&v)[8])
+{
+    uint4 q;
+    q.x = to_bf16(v[0]) | (to_bf16(v[1]) << 16);
+    q.y = to_bf16(v[2]) | (to_bf16(v[3]) << 16);
+    q.z = to_bf16(v[4]) | (to_bf16(v[5]) << 16);
+    q.w = to_bf16(v[6]) | (to_bf16(v[7]) << 16);
+    *(uint4 *)(sm.A + tc::tile_offset(row, 8 * part, 32)) = q;
+}
+
+// -log q(a | o) = log 2 + log f'(f^{-1}(a)) for the spline whose knots and
+// derivatives are in sm, and its gradient at the bin's knots and derivatives:
+// implicit differentiation of f(z) = a at fixed a (binary32; the same formulas
+// as the binary64 reference).
+__device__ __forceinline__ void nll_at_knots(Smem &sm, int row, float a)
 {
     constexpr int K = learned::kBins;
-    float prob[2][K], kn[2][K + 1], d[K + 1];
-    for (int part = 0; part < 2; ++part) {
-        const float *oo = o + part * K;
-        float mx = oo[0];
-        for (int i = 1; i < K; ++i) mx = fmaxf(mx, oo[i]);
-        float sum = 0.0f;
-        for (int i = 0; i < K; ++i) {
-            prob[part][i] = learned::exp_neg(oo[i] - mx);
-            sum += prob[part][i];
-        }
-        kn[part][0] = -1.0f;
-        for (int i = 0; i < K; ++i) {
-            prob[part][i] = prob[part][i] / sum;
-            kn[part][i + 1] = kn[part][i] + 2.0f * (learned::kMinBin + (1.0f - K * learned::kMinBin) * prob[part][i]);
-        }
-    }
-    for (int i = 0; i <= K; ++i) d[i] = learned::kMinDer + learned::softplus(o[2 * K + i]);
-    const float *x = kn[0], *y = kn[1];
     int k = 0;
+#pragma unroll
     for (int j = 1; j < K; ++j)
-        if (y[j] <= a) k = j;
-    const float W = x[k + 1] - x[k], H = y[k + 1] - y[k], D0 = d[k], D1 = d[k + 1];
-    const float s = H / W, dy = a - y[k], sig = D1 + D0 - 2.0f * s;
+        if (sm.knot[1][j][row] <= a) k = j;
+    const float xk = sm.knot[0][k][row], yk = sm.knot[1][k][row];
+    const float W = sm.knot[0][k + 1][row] - xk, H = sm.knot[1][k + 1][row] - yk;
+    const float D0 = sm.der[k][row], D1 = sm.der[k + 1][row];
+    const float s = H / W, dy = a - yk, sig = D1 + D0 - 2.0f * s;
     const float al = H * (s - D0) + dy * sig, be = H * D0 - dy * sig, c = -s * dy;
     const float disc = fmaxf(be * be - 4.0f * al * c, 0.0f);
     const float den_q = -be - sqrtf(disc);
@@ -169,120 +263,141 @@ __device__ float nll_and_grad(const float (&o)[learned::kOut], float a, float (&
     const float dY = -r;
     const float dHd = -r * (N / Dn);
     const float ds = (2.0f / s + 2.0f * t / M - 2.0f * (1.0f - 2.0f * t) / Dn) - r * F_s;
-    const float dD0 = ((1.0f - xi) * (1.0f - xi) / M - 2.0f * t / Dn) - r * F_D0;
-    const float dD1 = (xi * xi / M - 2.0f * t / Dn) - r * F_D1;
+    sm.g_der[0][row] = ((1.0f - xi) * (1.0f - xi) / M - 2.0f * t / Dn) - r * F_D0;
+    sm.g_der[1][row] = (xi * xi / M - 2.0f * t / Dn) - r * F_D1;
     const float dH = dHd + ds / W, dW = -ds * H / (W * W);
-    float gk[2][K + 1];
-    for (int i = 0; i <= K; ++i) gk[0][i] = gk[1][i] = 0.0f;
-    gk[1][k] += dY - dH;
-    gk[1][k + 1] += dH;
-    gk[0][k] -= dW;
-    gk[0][k + 1] += dW;
-    for (int part = 0; part < 2; ++part) {
-        float gw[K], dot = 0.0f, tail = 0.0f;
-        for (int i = K - 1; i >= 0; --i) {
-            tail += gk[part][i + 1];
-            gw[i] = tail * 2.0f * (1.0f - K * learned::kMinBin);
-        }
-        for (int i = 0; i < K; ++i) dot += gw[i] * prob[part][i];
-        for (int m = 0; m < K; ++m) g[part * K + m] = prob[part][m] * (gw[m] - dot);
-    }
-    for (int i = 0; i <= K; ++i) {
-        const float ti = o[2 * K + i];
-        const float sg = ti >= 0.0f ? 1.0f / (1.0f + learned::exp_neg(-ti)) : learned::exp_neg(ti) / (1.0f + learned::exp_neg(ti));
-        g[2 * K + i] = (i == k ? dD0 : (i == k + 1 ? dD1 : 0.0f)) * sg;
-    }
-    return 0.69314718f + L;
+    sm.g_knot[0][0][row] = 0.0f - dW;
+    sm.g_knot[0][1][row] = dW;
+    sm.g_knot[1][0][row] = dY - dH;
+    sm.g_knot[1][1][row] = dH;
+    sm.bin[row] = k;
+    sm.loss[row] = 0.69314718f + L;
 }
 
-struct StepParams {
-    const float *w;            // 1947 master weights (fp32)
-    const float2 *pairs;       // (beta k, a0)
-    long long n_pairs;
-    int explicit_rows;         // 1: row r of CTA b is pair b*128 + r; 0: random pairs
-    uint32_t step, k0, k1;     // Philox key and counter for random pairs
-    float *partials;           // [gridDim.x][kGradSlots]
-    unsigned int *err;
-};
-
-__device__ __forceinline__ uint16_t to_bf16(float f)
+// The likelihood of the sample and its gradient with respect to this thread's
+// network outputs o (part 0: log widths, 1: log heights, 2 and 3: the
+// unconstrained derivatives), through the knot sums and the softmax or the
+// softplus.  Every thread calls it (barriers inside).
+__device__ __forceinline__ void nll_and_grad(Smem &sm, int row, int part, float a, const float (&o)[8], float (&g)[8])
 {
-    const uint32_t u = __float_as_uint(f);
-    return (uint16_t)((u + 0x7FFFu + ((u >> 16) & 1u)) >> 16);
-}
-
-struct Smem {
-    unsigned char A[kRows * 32 * 2];     // activation tile (A operand)
-    unsigned char W2[32 * 32 * 2];       // B: W2 (n = output j, k = input i)
-    unsigned char W3[32 * 32 * 2];       // B: W3 (n = output o, padded to 32)
-    unsigned char W3T[32 * 32 * 2];      // B: W3^T (n = j, k = o padded)
-    unsigned char W2T[32 * 32 * 2];      // B: W2^T (n = i, k = j)
-    float h1[kRows][kPad], h2[kRows][kPad], go[kRows][kPad], dz2[kRows][kPad], dz1[kRows][kPad];
-    float s_in[kRows];
-    float loss[kRows];
-    uint64_t mbar;
-    uint32_t tmem_base;
-};
-
-// One MMA pass: D (tmem) = A (smem tile, 128 x 32) * B^T (32 x 32), then this
-// thread's row of D into v.  Every thread must call it (barriers inside).
-__device__ bool mma_pass(Smem &sm, const unsigned char *B, uint32_t taddr, uint32_t &phase, float (&v)[32])
-{
-    tc::fence_smem_to_async();
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    if (threadIdx.x == 0) {
-        const uint32_t idesc = tc::idesc_bf16_f32(128, 32);
-        for (int j = 0; j < 2; ++j) {
-            const uint64_t ad = tc::smem_desc(tc::smem_addr(sm.A) + 256u * j, 128u, 512u);
-            const uint64_t bd = tc::smem_desc(tc::smem_addr(B) + 256u * j, 128u, 512u);
-            tc::mma_bf16(taddr, ad, bd, idesc, j > 0 ? 1u : 0u);
-        }
-        tc::mma_commit(&sm.mbar);
-    }
-    bool ok = tc::mbar_wait(&sm.mbar, phase, kMbarPolls);
-    if (!ok) ok = tc::mbar_wait(&sm.mbar, phase, kMbarPolls);
-    phase ^= 1u;
-    tc::fence_after_sync();
-    if (ok) {
-        tc::tmem_load32(taddr + ((uint32_t)((threadIdx.x >> 5) * 32) << 16), v);
-    } else {
+    constexpr int K = learned::kBins;
+    float q[8];  // parts 0, 1: softmax probabilities; 2, 3: the derivatives' sigmoids
+    if (part < 2) {
+        float mx = o[0];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = 0.0f;
+        for (int i = 1; i < K; ++i) mx = fmaxf(mx, o[i]);
+        float sum = 0.0f;
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            q[i] = learned::exp_neg(o[i] - mx);
+            sum += q[i];
+        }
+        float kn = -1.0f;
+        sm.knot[part][0][row] = kn;
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            q[i] = q[i] / sum;
+            kn = kn + 2.0f * (learned::kMinBin + (1.0f - K * learned::kMinBin) * q[i]);
+            sm.knot[part][i + 1][row] = kn;
+        }
+    } else {
+        const int n = part == 2 ? 8 : 1;  // warp-uniform
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            q[i] = 0.0f;
+            if (i < n) {
+                const float e = learned::exp_neg(o[i] < 0.0f ? o[i] : -o[i]);
+                const float one_e = 1.0f + e;
+                sm.der[8 * (part - 2) + i][row] = learned::kMinDer + ((o[i] > 0.0f ? o[i] : 0.0f) + log_series(one_e));
+                q[i] = o[i] >= 0.0f ? 1.0f / one_e : e / one_e;
+            }
+        }
     }
-    tc::fence_before_sync();
-    __syncthreads();  // every thread has read D and A before either is overwritten
-    return ok;
+    __syncthreads();
+    if (part == 0) nll_at_knots(sm, row, a);
+    __syncthreads();
+    const int k = sm.bin[row];
+    if (part < 2) {
+        // sums of the knots' gradients above each bin: none, k + 1's, both
+        const float g1 = 0.0f + sm.g_knot[part][1][row], g01 = g1 + sm.g_knot[part][0][row];
+        float dot = 0.0f;
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            g[i] = (i > k ? 0.0f : (i == k ? g1 : g01)) * 2.0f * (1.0f - K * learned::kMinBin);
+            dot += g[i] * q[i];
+        }
+#pragma unroll
+        for (int i = 0; i < K; ++i) g[i] = q[i] * (g[i] - dot);
+    } else {
+        const float d0 = sm.g_der[0][row], d1 = sm.g_der[1][row];
+        const int first = 8 * (part - 2);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) g[i] = (first + i == k ? d0 : (first + i == k + 1 ? d1 : 0.0f)) * q[i];
+    }
 }
 
-__device__ __forceinline__ void put_row_bf16(Smem &sm, int row, const float *vals, int n)
+// Sum over the rows, in order, of f(r): four products at a time.
+__device__ __forceinline__ float4 row_products(const float (&lhs)[kRows][kPitch], int j4, const float (&rhs)[kRows][kPitch],
+                                               int col)
 {
-    for (int k = 0; k < 32; ++k) *(uint16_t *)(sm.A + tc::tile_offset(row, k, 32)) = k < n ? to_bf16(vals[k]) : (uint16_t)0;
+    float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll 8
+    for (int r = 0; r < kRows; ++r) {
+        const float4 d = *(const float4 *)&lhs[r][j4];
+        const float x = rhs[r][col];
+        acc.x += d.x * x;
+        acc.y += d.y * x;
+        acc.z += d.z * x;
+        acc.w += d.w * x;
+    }
+    return acc;
 }
 
 // Forward + backward of kRows samples per CTA; per-CTA sums of the 1945
 // gradients and of the loss go to partials[blockIdx.x].
-__global__ void __launch_bounds__(kRows) train_step_kernel(const StepParams p)
+__global__ void __launch_bounds__(kTrainThreads) train_step_kernel(const StepParams p)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
-    const int t = threadIdx.x, warp = t >> 5;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int row = t & (kRows - 1), part = t >> 7;
     const float *w = p.w;
 
-    // B operands (bf16, core-matrix layout)
-    for (int q = t; q < 32 * 32; q += blockDim.x) {
-        const int r = q >> 5, c = q & 31;
-        *(uint16_t *)(sm.W2 + tc::tile_offset(r, c, 32)) = to_bf16(w[learned::kOffW2 + r * 32 + c]);
-        *(uint16_t *)(sm.W2T + tc::tile_offset(r, c, 32)) = to_bf16(w[learned::kOffW2 + c * 32 + r]);
-        *(uint16_t *)(sm.W3 + tc::tile_offset(r, c, 32)) = r < learned::kOut ? to_bf16(w[learned::kOffW3 + r * 32 + c]) : (uint16_t)0;
-        *(uint16_t *)(sm.W3T + tc::tile_offset(r, c, 32)) = c < learned::kOut ? to_bf16(w[learned::kOffW3 + c * 32 + r]) : (uint16_t)0;
-    }
+    // what does not depend on the weights: tensor memory, the barrier, the sample
+    release_next_grid();
     if (warp == 0) tc::tmem_alloc(&sm.tmem_base, 32);
     if (t == 0) {
         tc::mbar_init(&sm.mbar, 1);
         mbar_init_fence();
     }
+    long long idx;
+    if (p.explicit_rows) {
+        idx = (long long)blockIdx.x * kRows + row;
+    } else {
+        const uint4 r = philox_key(make_uint4((uint32_t)(blockIdx.x * kRows + row), p.step, 5u << 3, 0u), p.k0, p.k1);
+        idx = (long long)(((unsigned long long)r.x * (unsigned long long)p.n_pairs) >> 32);
+    }
+    const float2 pr = p.pairs[idx];
+    wait_previous_grid();
+
+    // B operands (bf16, core-matrix layout); W3 padded to 32 rows with zeros
+#pragma unroll
+    for (int q = t; q < 32 * 32; q += kTrainThreads) {
+        const int r = q >> 5, c = q & 31;
+        const uint16_t w2 = (uint16_t)to_bf16(w[learned::kOffW2 + q]);
+        const uint16_t w3 = r < learned::kOut ? (uint16_t)to_bf16(w[learned::kOffW3 + q]) : (uint16_t)0;
+        *(uint16_t *)(sm.W2 + tc::tile_offset(r, c, 32)) = w2;
+        *(uint16_t *)(sm.W2T + tc::tile_offset(c, r, 32)) = w2;
+        *(uint16_t *)(sm.W3 + tc::tile_offset(r, c, 32)) = w3;
+        *(uint16_t *)(sm.W3T + tc::tile_offset(c, r, 32)) = w3;
+    }
+    if (warp == 0) sm.w1[lane] = w[learned::kOffW1 + lane];
+    if (warp == 1) sm.b1[lane] = w[learned::kOffB1 + lane];
+    if (warp == 2) sm.b2[lane] = w[learned::kOffB2 + lane];
+    if (warp == 3) sm.b3[lane] = lane < learned::kOut ? w[learned::kOffB3 + lane] : 0.0f;
+    const float s = (pr.x - w[learned::kOffMean]) * w[learned::kOffScale];
+    const float a = fminf(fmaxf(pr.y, -1.0f), 1.0f);
+    if (part == 0) sm.s_in[row] = s;
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -290,72 +405,79 @@ __global__ void __launch_bounds__(kRows) train_step_kernel(const StepParams p)
     uint32_t phase = 0;
     bool ok = true;
 
-    // sample of this row
-    long long idx;
-    if (p.explicit_rows) {
-        idx = (long long)blockIdx.x * kRows + t;
-    } else {
-        const uint4 r = philox_key(make_uint4((uint32_t)(blockIdx.x * kRows + t), p.step, 5u << 3, 0u), p.k0, p.k1);
-        idx = (long long)(((unsigned long long)r.x * (unsigned long long)p.n_pairs) >> 32);
-    }
-    const float2 pr = p.pairs[idx];
-    const float s = (pr.x - w[learned::kOffMean]) * w[learned::kOffScale];
-    const float a = fminf(fmaxf(pr.y, -1.0f), 1.0f);
-    sm.s_in[t] = s;
-
     // layer 1 (fp32), layer 2 (tensor cores)
-    float v[32];
-    for (int j = 0; j < 32; ++j) v[j] = learned::relu(w[learned::kOffW1 + j] * s + w[learned::kOffB1 + j]);
-    for (int j = 0; j < 32; ++j) sm.h1[t][j] = v[j];
-    put_row_bf16(sm, t, v, 32);
+    const int c0 = 8 * part;
+    float v[8], h1[8], h2[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) h1[j] = learned::relu(sm.w1[c0 + j] * s + sm.b1[c0 + j]);
+    stash_row(sm.h1, row, part, h1);
+    put_row_bf16(sm, row, part, h1);
     ok &= mma_pass(sm, sm.W2, taddr, phase, v);
-    for (int j = 0; j < 32; ++j) v[j] = learned::relu(v[j] + w[learned::kOffB2 + j]);
-    for (int j = 0; j < 32; ++j) sm.h2[t][j] = v[j];
-    put_row_bf16(sm, t, v, 32);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) h2[j] = learned::relu(v[j] + sm.b2[c0 + j]);
+    stash_row(sm.h2, row, part, h2);
+    put_row_bf16(sm, row, part, h2);
     // layer 3 (tensor cores)
     ok &= mma_pass(sm, sm.W3, taddr, phase, v);
-    float o[learned::kOut], go[learned::kOut];
-    for (int j = 0; j < learned::kOut; ++j) o[j] = v[j] + w[learned::kOffB3 + j];
-    sm.loss[t] = nll_and_grad(o, a, go);
-    for (int j = 0; j < 32; ++j) sm.go[t][j] = j < learned::kOut ? go[j] : 0.0f;
-    put_row_bf16(sm, t, go, learned::kOut);
+    float go[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = v[j] + sm.b3[c0 + j];
+    nll_and_grad(sm, row, part, a, v, go);
+    stash_row(sm.go, row, part, go);
+    put_row_bf16(sm, row, part, go);
     // dh2 = go W3 (tensor cores), through the ReLU
     ok &= mma_pass(sm, sm.W3T, taddr, phase, v);
-    for (int j = 0; j < 32; ++j) v[j] = sm.h2[t][j] > 0.0f ? v[j] : 0.0f;
-    for (int j = 0; j < 32; ++j) sm.dz2[t][j] = v[j];
-    put_row_bf16(sm, t, v, 32);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = h2[j] > 0.0f ? v[j] : 0.0f;
+    stash_row(sm.dz2, row, part, v);
+    put_row_bf16(sm, row, part, v);
     // dh1 = dz2 W2 (tensor cores), through the ReLU
     ok &= mma_pass(sm, sm.W2T, taddr, phase, v);
-    for (int j = 0; j < 32; ++j) sm.dz1[t][j] = sm.h1[t][j] > 0.0f ? v[j] : 0.0f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = h1[j] > 0.0f ? v[j] : 0.0f;
+    stash_row(sm.dz1, row, part, v);
     if (!ok && t == 0) atomicAdd(p.err, 1u);
-    __syncthreads();
-
-    // per-CTA gradient sums (fp32, rows in order)
-    float *out = p.partials + (size_t)blockIdx.x * kGradSlots;
-    for (int q = t; q < kGradSlots; q += blockDim.x) {
-        float acc = 0.0f;
-        if (q < 32) {  // W1
-            for (int r = 0; r < kRows; ++r) acc += sm.dz1[r][q] * sm.s_in[r];
-        } else if (q < 64) {  // b1
-            for (int r = 0; r < kRows; ++r) acc += sm.dz1[r][q - 32];
-        } else if (q < 1088) {  // W2[j][i]
-            const int j = (q - 64) >> 5, i = (q - 64) & 31;
-            for (int r = 0; r < kRows; ++r) acc += sm.dz2[r][j] * sm.h1[r][i];
-        } else if (q < 1120) {  // b2
-            for (int r = 0; r < kRows; ++r) acc += sm.dz2[r][q - 1088];
-        } else if (q < 1920) {  // W3[o][j]
-            const int oo = (q - 1120) >> 5, j = (q - 1120) & 31;
-            for (int r = 0; r < kRows; ++r) acc += sm.go[r][oo] * sm.h2[r][j];
-        } else if (q < 1945) {  // b3
-            for (int r = 0; r < kRows; ++r) acc += sm.go[r][q - 1920];
-        } else {  // loss
-            for (int r = 0; r < kRows; ++r) acc += sm.loss[r];
-        }
-        out[q] = acc;
-    }
     tc::fence_before_sync();
     __syncthreads();
     if (warp == 0) tc::tmem_dealloc(taddr, 32);
+
+    // per-CTA gradient sums (fp32, rows in order): warps 0..7 four rows of W2
+    // each, 8..14 four rows of W3, 15 the vectors
+    float *out = p.partials + (size_t)blockIdx.x * kGradSlots;
+    if (warp < 8) {
+        const float4 g = row_products(sm.dz2, 4 * warp, sm.h1, lane);
+        float *const to = out + learned::kOffW2 + 128 * warp + lane;
+        to[0] = g.x;
+        to[32] = g.y;
+        to[64] = g.z;
+        to[96] = g.w;
+    } else if (warp < 15) {
+        const int o0 = 4 * (warp - 8);
+        const float4 g = row_products(sm.go, o0, sm.h2, lane);
+        float *const to = out + learned::kOffW3 + 32 * o0 + lane;
+        to[0] = g.x;
+        if (o0 + 1 < learned::kOut) {
+            to[32] = g.y;
+            to[64] = g.z;
+            to[96] = g.w;
+        }
+    } else {
+        float w1 = 0.0f, b1 = 0.0f, b2 = 0.0f, b3 = 0.0f, loss = 0.0f;
+#pragma unroll 8
+        for (int r = 0; r < kRows; ++r) {
+            const float d = sm.dz1[r][lane];
+            w1 += d * sm.s_in[r];
+            b1 += d;
+            b2 += sm.dz2[r][lane];
+            b3 += sm.go[r][lane];
+            loss += sm.loss[r];
+        }
+        out[learned::kOffW1 + lane] = w1;
+        out[learned::kOffB1 + lane] = b1;
+        out[learned::kOffB2 + lane] = b2;
+        if (lane < learned::kOut) out[learned::kOffB3 + lane] = b3;
+        if (lane == 0) out[learned::kTrainable] = loss;
+    }
 }
 
 // Sums the per-CTA partials (in CTA order) into the mean gradient and loss;
@@ -366,8 +488,11 @@ __global__ void adam_kernel(float *__restrict__ w, float *__restrict__ m, float 
                             float *__restrict__ loss_out)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    release_next_grid();
+    wait_previous_grid();
     if (i >= kGradSlots) return;
     float gsum = 0.0f;
+#pragma unroll 16
     for (int b = 0; b < nblocks; ++b) gsum += partials[(size_t)b * kGradSlots + i];
     const float g = gsum * inv_batch;
     if (i == learned::kTrainable) {
@@ -384,31 +509,49 @@ __global__ void adam_kernel(float *__restrict__ w, float *__restrict__ m, float 
     }
 }
 
-// mean and 1 / standard deviation of beta k over the pairs -> w[1945], w[1946]
-__global__ void input_scaling_kernel(const float2 *__restrict__ pairs, long long n, float *__restrict__ w)
+// mean and 1 / standard deviation of beta k over the pairs -> w[1945],
+// w[1946]: block sums in binary64, added in block order by the block that
+// finishes last (the ticket returns to 0).  One block for all pairs waited
+// for its loads 780 times over 200,000 pairs (255 us under ncu); with a block
+// per 2048 pairs, up to one per SM, SCALING_FIGURES
+constexpr int kScalingThreads = 256;
+
+__global__ void __launch_bounds__(kScalingThreads)
+    input_scaling_kernel(const float2 *__restrict__ pairs, long long n, double *__restrict__ sums,
+                         unsigned int *__restrict__ ticket, float *__restrict__ w)
 {
-    __shared__ double s1[256], s2[256];
     double a = 0.0, b = 0.0;
-    for (long long i = threadIdx.x; i < n; i += blockDim.x) {
+#pragma unroll 4
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const double x = (double)pairs[i].x;
         a += x;
         b += x * x;
     }
-    s1[threadIdx.x] = a;
-    s2[threadIdx.x] = b;
-    __syncthreads();
-    for (int off = blockDim.x / 2; off > 0; off >>= 1) {
-        if (threadIdx.x < off) {
-            s1[threadIdx.x] += s1[threadIdx.x + off];
-            s2[threadIdx.x] += s2[threadIdx.x + off];
-        }
-        __syncthreads();
-    }
+    a = block_sum(a);
+    b = block_sum(b);
+    __shared__ bool last;
     if (threadIdx.x == 0) {
-        const double mean = s1[0] / (double)n;
-        const double var = s2[0] / (double)n - mean * mean;
+        sums[2 * blockIdx.x] = a;
+        sums[2 * blockIdx.x + 1] = b;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    a = b = 0.0;
+    for (unsigned int i = threadIdx.x; i < gridDim.x; i += blockDim.x) {
+        a += ((volatile double *)sums)[2 * i];
+        b += ((volatile double *)sums)[2 * i + 1];
+    }
+    a = block_sum(a);
+    b = block_sum(b);
+    if (threadIdx.x == 0) {
+        const double mean = a / (double)n;
+        const double var = b / (double)n - mean * mean;
         w[learned::kOffMean] = (float)mean;
         w[learned::kOffScale] = (float)(1.0 / sqrt(var > 1e-12 ? var : 1e-12));
+        *ticket = 0u;
     }
 }
 
@@ -423,7 +566,7 @@ struct su2_trainer {
     void *block = nullptr;
     size_t block_bytes = 0;
     float *w = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr, *loss = nullptr;
-    unsigned int *err = nullptr;
+    unsigned int *err = nullptr;  // [0] waits given up, [16] ticket of the input scaling
     float *partials = nullptr;
     int partial_blocks = 0;
     float *losses = nullptr;  // per step of the last fit
@@ -434,6 +577,26 @@ namespace su2 {
 namespace {
 
 constexpr int kMaxBatch = 65536;
+
+// Launches a kernel whose prologue may overlap the tail of the previous kernel
+// of the stream (it waits with griddepcontrol.wait before it touches anything
+// that one writes).
+template <typename... Args>
+cudaError_t launch_dependent(void (*kernel)(Args...), int grid, int threads, size_t smem, cudaStream_t stream,
+                             Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 
 su2_status trainer_launch(su2_trainer *tr, const float *pairs, long long n, int batch, int explicit_rows, float lr,
                           float *loss_dst)
@@ -449,18 +612,17 @@ su2_status trainer_launch(su2_trainer *tr, const float *pairs, long long n, int 
     p.k1 = (uint32_t)(tr->seed >> 32);
     p.partials = tr->partials;
     p.err = tr->err;
-    train::train_step_kernel<<<nblocks, train::kRows, sizeof(train::Smem), tr->stream>>>(p);
-    SU2_CUDA(cudaGetLastError());
+    SU2_CUDA(launch_dependent(train::train_step_kernel, nblocks, train::kTrainThreads, sizeof(train::Smem), tr->stream,
+                              p));
     float bias1 = 1.0f, bias2 = 1.0f;
     if (lr > 0.0f) {
         tr->step += 1;
         bias1 = 1.0f - powf(0.9f, (float)tr->step);
         bias2 = 1.0f - powf(0.999f, (float)tr->step);
     }
-    train::adam_kernel<<<(train::kGradSlots + 255) / 256, 256, 0, tr->stream>>>(
-        tr->w, tr->m, tr->v, tr->partials, nblocks, 1.0f / (float)batch, lr, 0.9f, 0.999f, 1e-8f, bias1, bias2,
-        tr->grad, loss_dst);
-    SU2_CUDA(cudaGetLastError());
+    SU2_CUDA(launch_dependent(train::adam_kernel, (train::kGradSlots + 63) / 64, 64, 0, tr->stream, tr->w, tr->m, tr->v,
+                              (const float *)tr->partials, nblocks, 1.0f / (float)batch, lr, 0.9f, 0.999f, 1e-8f, bias1,
+                              bias2, tr->grad, loss_dst));
     return SU2_OK;
 }
 
@@ -543,7 +705,12 @@ su2_status su2_trainer_set_input_scaling(su2_trainer *tr, const float *dev_pairs
 {
     if (!tr || !dev_pairs || n < 2) return SU2_E_INVAL;
     DeviceGuard guard(tr->device);
-    train::input_scaling_kernel<<<1, 256, 0, tr->stream>>>((const float2 *)dev_pairs, (long long)n, tr->w);
+    // the block sums take the head of the step partials, idle between calls
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, tr->device);
+    const int grid = (int)std::min<size_t>((n + 2047) / 2048, (size_t)sms);
+    train::input_scaling_kernel<<<grid, train::kScalingThreads, 0, tr->stream>>>(
+        (const float2 *)dev_pairs, (long long)n, (double *)tr->partials, tr->err + 16, tr->w);
     SU2_CUDA(cudaGetLastError());
     SU2_CUDA(cudaStreamSynchronize(tr->stream));
     return SU2_OK;
