@@ -126,7 +126,9 @@ namespace train {
 // The gradient sums over the 128 rows (rows in order, binary32) take all 16
 // warps, four outputs per thread: one 16-byte broadcast and one conflict-free
 // load per four multiply-adds.  Batches of 4096 fill 32 SMs with one CTA each,
-// so a step is latency, not throughput: TRAIN_FIGURES
+// so a step is latency, not throughput.  One thread per sample
+// took 39.6 us under ncu, this 12.9; a step with its Adam update 33 -> 12 us
+// in a fit.
 constexpr int kRows = 128;                   // samples per CTA
 constexpr int kParts = 4;                    // threads per sample
 constexpr int kTrainThreads = kRows * kParts;
@@ -135,11 +137,13 @@ constexpr int kGradSlots = learned::kTrainable + 1;  // 1945 gradients + loss su
 
 struct StepParams {
     const float *w;            // 1947 master weights (fp32)
+    const uint4 *images;       // their BF16 operand tiles (put_images)
+    int split;                 // CTAs per 128 samples: 1, 2 or 4
     const float2 *pairs;       // (beta k, a0)
     long long n_pairs;
     int explicit_rows;         // 1: row r of CTA b is pair b*128 + r; 0: random pairs
     uint32_t step, k0, k1;     // Philox key and counter for random pairs
-    float *partials;           // [gridDim.x][kGradSlots]
+    float *partials;           // [gridDim.x / split][kGradSlots]
     unsigned int *err;
 };
 
@@ -149,18 +153,42 @@ __device__ __forceinline__ uint32_t to_bf16(float f)
     return (u + 0x7FFFu + ((u >> 16) & 1u)) >> 16;
 }
 
+// The B operands as the tensor cores take them (BF16, core-matrix layout): W2
+// (n = output j, k = input i), W3 (n = output o, padded to 32), W3^T (n = j,
+// k = o padded), W2^T (n = i, k = j), 2 KB each.  Kept beside the master
+// weights (the Adam kernel writes both), so a CTA fetches them as one 16-byte
+// load per thread instead of converting and scattering 1824 weights.
+constexpr uint32_t kTileBytes = 32 * 32 * 2;
+constexpr uint32_t kImageBytes = 4 * kTileBytes;
+static_assert(kImageBytes == 16 * kTrainThreads, "one 16-byte load per thread");
+
+__device__ __forceinline__ void put_images(unsigned char *images, int i, float w)
+{
+    const bool w2 = i >= learned::kOffW2 && i < learned::kOffB2;
+    if (!w2 && !(i >= learned::kOffW3 && i < learned::kOffB3)) return;
+    const int q = i - (w2 ? learned::kOffW2 : learned::kOffW3);
+    const int r = q >> 5, c = q & 31;
+    const uint16_t h = (uint16_t)to_bf16(w);
+    *(uint16_t *)(images + (w2 ? 0 : kTileBytes) + tc::tile_offset(r, c, 32)) = h;
+    *(uint16_t *)(images + (w2 ? 3 * kTileBytes : 2 * kTileBytes) + tc::tile_offset(c, r, 32)) = h;
+}
+
+__global__ void put_images_kernel(const float *__restrict__ w, unsigned char *__restrict__ images)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < learned::kTrainable) put_images(images, i, w[i]);
+}
+
 struct Smem {
     unsigned char A[kRows * 32 * 2];     // activation tile (A operand)
-    unsigned char W2[32 * 32 * 2];       // B: W2 (n = output j, k = input i)
-    unsigned char W3[32 * 32 * 2];       // B: W3 (n = output o, padded to 32)
-    unsigned char W3T[32 * 32 * 2];      // B: W3^T (n = j, k = o padded)
-    unsigned char W2T[32 * 32 * 2];      // B: W2^T (n = i, k = j)
+    unsigned char W2[kTileBytes], W3[kTileBytes], W3T[kTileBytes], W2T[kTileBytes];  // B operands
     float h1[kRows][kPitch], h2[kRows][kPitch], go[kRows][kPitch], dz2[kRows][kPitch], dz1[kRows][kPitch];
     float w1[32], b1[32], b2[32], b3[32];
     float knot[2][learned::kBins + 1][kRows];  // x_0 .. x_8, y_0 .. y_8 of each sample
     float der[learned::kBins + 1][kRows];
     float g_knot[2][2][kRows];           // gradient at knots k, k + 1 of x and y
     float g_der[2][kRows];               // gradient at derivatives k, k + 1
+    float handed_o[3][kRows], handed_q[3][kRows];  // derivatives 5 .. 7: outputs to part 3, sigmoids back
     int bin[kRows];
     float s_in[kRows];
     float loss[kRows];
@@ -282,6 +310,11 @@ __device__ __forceinline__ void nll_and_grad(Smem &sm, int row, int part, float 
 {
     constexpr int K = learned::kBins;
     float q[8];  // parts 0, 1: softmax probabilities; 2, 3: the derivatives' sigmoids
+    if (part == 2) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) sm.handed_o[i][row] = o[5 + i];
+    }
+    __syncthreads();
     if (part < 2) {
         float mx = o[0];
 #pragma unroll
@@ -301,16 +334,32 @@ __device__ __forceinline__ void nll_and_grad(Smem &sm, int row, int part, float 
             sm.knot[part][i + 1][row] = kn;
         }
     } else {
-        const int n = part == 2 ? 8 : 1;  // warp-uniform
+        // five derivatives in part 2, four in part 3 (three of them handed over)
+        const int n = part == 2 ? 5 : 4;  // warp-uniform
+        float od[5] = {o[0], o[1], o[2], o[3], o[4]};
+        if (part == 3) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            q[i] = 0.0f;
+            for (int i = 0; i < 3; ++i) od[i] = sm.handed_o[i][row];
+            od[3] = o[0];
+        }
+        float sg[5];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            sg[i] = 0.0f;
             if (i < n) {
-                const float e = learned::exp_neg(o[i] < 0.0f ? o[i] : -o[i]);
+                const float e = learned::exp_neg(od[i] < 0.0f ? od[i] : -od[i]);
                 const float one_e = 1.0f + e;
-                sm.der[8 * (part - 2) + i][row] = learned::kMinDer + ((o[i] > 0.0f ? o[i] : 0.0f) + log_series(one_e));
-                q[i] = o[i] >= 0.0f ? 1.0f / one_e : e / one_e;
+                sm.der[5 * (part - 2) + i][row] =
+                    learned::kMinDer + ((od[i] > 0.0f ? od[i] : 0.0f) + log_series(one_e));
+                sg[i] = od[i] >= 0.0f ? 1.0f / one_e : e / one_e;
             }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) q[i] = part == 2 && i < 5 ? sg[i] : 0.0f;
+        if (part == 3) {
+#pragma unroll
+            for (int i = 0; i < 3; ++i) sm.handed_q[i][row] = sg[i];
+            q[0] = sg[3];
         }
     }
     __syncthreads();
@@ -329,6 +378,10 @@ __device__ __forceinline__ void nll_and_grad(Smem &sm, int row, int part, float 
 #pragma unroll
         for (int i = 0; i < K; ++i) g[i] = q[i] * (g[i] - dot);
     } else {
+        if (part == 2) {
+#pragma unroll
+            for (int i = 0; i < 3; ++i) q[5 + i] = sm.handed_q[i][row];
+        }
         const float d0 = sm.g_der[0][row], d1 = sm.g_der[1][row];
         const int first = 8 * (part - 2);
 #pragma unroll
@@ -353,8 +406,11 @@ __device__ __forceinline__ float4 row_products(const float (&lhs)[kRows][kPitch]
     return acc;
 }
 
-// Forward + backward of kRows samples per CTA; per-CTA sums of the 1945
-// gradients and of the loss go to partials[blockIdx.x].
+// Forward + backward of kRows samples; their sums of the 1945 gradients and of
+// the loss go to partials[block].  `split` CTAs run the same samples, each
+// adding its share of the gradients: where the batch leaves SMs idle, the
+// sums (the longest stage, 7.8 of 28 thousand cycles in one CTA) shrink with
+// the split while the repeated forward pass costs nothing.
 __global__ void __launch_bounds__(kTrainThreads) train_step_kernel(const StepParams p)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -370,27 +426,18 @@ __global__ void __launch_bounds__(kTrainThreads) train_step_kernel(const StepPar
         tc::mbar_init(&sm.mbar, 1);
         mbar_init_fence();
     }
+    const int block = (int)blockIdx.x / p.split;
     long long idx;
     if (p.explicit_rows) {
-        idx = (long long)blockIdx.x * kRows + row;
+        idx = (long long)block * kRows + row;
     } else {
-        const uint4 r = philox_key(make_uint4((uint32_t)(blockIdx.x * kRows + row), p.step, 5u << 3, 0u), p.k0, p.k1);
+        const uint4 r = philox_key(make_uint4((uint32_t)(block * kRows + row), p.step, 5u << 3, 0u), p.k0, p.k1);
         idx = (long long)(((unsigned long long)r.x * (unsigned long long)p.n_pairs) >> 32);
     }
     const float2 pr = p.pairs[idx];
     wait_previous_grid();
 
-    // B operands (bf16, core-matrix layout); W3 padded to 32 rows with zeros
-#pragma unroll
-    for (int q = t; q < 32 * 32; q += kTrainThreads) {
-        const int r = q >> 5, c = q & 31;
-        const uint16_t w2 = (uint16_t)to_bf16(w[learned::kOffW2 + q]);
-        const uint16_t w3 = r < learned::kOut ? (uint16_t)to_bf16(w[learned::kOffW3 + q]) : (uint16_t)0;
-        *(uint16_t *)(sm.W2 + tc::tile_offset(r, c, 32)) = w2;
-        *(uint16_t *)(sm.W2T + tc::tile_offset(c, r, 32)) = w2;
-        *(uint16_t *)(sm.W3 + tc::tile_offset(r, c, 32)) = w3;
-        *(uint16_t *)(sm.W3T + tc::tile_offset(c, r, 32)) = w3;
-    }
+    ((uint4 *)sm.W2)[t] = p.images[t];
     if (warp == 0) sm.w1[lane] = w[learned::kOffW1 + lane];
     if (warp == 1) sm.b1[lane] = w[learned::kOffB1 + lane];
     if (warp == 2) sm.b2[lane] = w[learned::kOffB2 + lane];
@@ -441,18 +488,21 @@ __global__ void __launch_bounds__(kTrainThreads) train_step_kernel(const StepPar
     __syncthreads();
     if (warp == 0) tc::tmem_dealloc(taddr, 32);
 
-    // per-CTA gradient sums (fp32, rows in order): warps 0..7 four rows of W2
-    // each, 8..14 four rows of W3, 15 the vectors
-    float *out = p.partials + (size_t)blockIdx.x * kGradSlots;
-    if (warp < 8) {
-        const float4 g = row_products(sm.dz2, 4 * warp, sm.h1, lane);
-        float *const to = out + learned::kOffW2 + 128 * warp + lane;
+    // gradient sums (fp32, rows in order), a warp per task: 0..7 four rows of
+    // W2 each, 8..14 four rows of W3, 15 the vectors
+    const int tasks = 16 / p.split;
+    if (warp >= tasks) return;
+    const int task = ((int)blockIdx.x - block * p.split) * tasks + warp;
+    float *out = p.partials + (size_t)block * kGradSlots;
+    if (task < 8) {
+        const float4 g = row_products(sm.dz2, 4 * task, sm.h1, lane);
+        float *const to = out + learned::kOffW2 + 128 * task + lane;
         to[0] = g.x;
         to[32] = g.y;
         to[64] = g.z;
         to[96] = g.w;
-    } else if (warp < 15) {
-        const int o0 = 4 * (warp - 8);
+    } else if (task < 15) {
+        const int o0 = 4 * (task - 8);
         const float4 g = row_products(sm.go, o0, sm.h2, lane);
         float *const to = out + learned::kOffW3 + 32 * o0 + lane;
         to[0] = g.x;
@@ -485,7 +535,7 @@ __global__ void __launch_bounds__(kTrainThreads) train_step_kernel(const StepPar
 __global__ void adam_kernel(float *__restrict__ w, float *__restrict__ m, float *__restrict__ v,
                             const float *__restrict__ partials, int nblocks, float inv_batch, float lr, float b1,
                             float b2, float eps, float bias1, float bias2, float *__restrict__ grad_out,
-                            float *__restrict__ loss_out)
+                            float *__restrict__ loss_out, unsigned char *__restrict__ images)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     release_next_grid();
@@ -505,7 +555,9 @@ __global__ void adam_kernel(float *__restrict__ w, float *__restrict__ m, float 
         const float vi = b2 * v[i] + (1.0f - b2) * g * g;
         m[i] = mi;
         v[i] = vi;
-        w[i] -= lr * (mi / bias1) / (sqrtf(vi / bias2) + eps);
+        const float wi = w[i] - lr * (mi / bias1) / (sqrtf(vi / bias2) + eps);
+        w[i] = wi;
+        put_images(images, i, wi);
     }
 }
 
@@ -513,7 +565,7 @@ __global__ void adam_kernel(float *__restrict__ w, float *__restrict__ m, float 
 // w[1946]: block sums in binary64, added in block order by the block that
 // finishes last (the ticket returns to 0).  One block for all pairs waited
 // for its loads 780 times over 200,000 pairs (255 us under ncu); with a block
-// per 2048 pairs, up to one per SM, SCALING_FIGURES
+// per 2048 pairs, up to one per SM, 13 us.
 constexpr int kScalingThreads = 256;
 
 __global__ void __launch_bounds__(kScalingThreads)
@@ -560,6 +612,7 @@ __global__ void __launch_bounds__(kScalingThreads)
 
 struct su2_trainer {
     int device = 0;
+    int sms = 0;
     cudaStream_t stream = nullptr;
     uint64_t seed = 0;
     uint32_t step = 0;  // Adam steps taken
@@ -567,6 +620,7 @@ struct su2_trainer {
     size_t block_bytes = 0;
     float *w = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr, *loss = nullptr;
     unsigned int *err = nullptr;  // [0] waits given up, [16] ticket of the input scaling
+    unsigned char *images = nullptr;  // BF16 operand tiles of w
     float *partials = nullptr;
     int partial_blocks = 0;
     float *losses = nullptr;  // per step of the last fit
@@ -604,6 +658,9 @@ su2_status trainer_launch(su2_trainer *tr, const float *pairs, long long n, int 
     const int nblocks = batch / train::kRows;
     train::StepParams p;
     p.w = tr->w;
+    p.images = (const uint4 *)tr->images;
+    // CTAs per 128 samples: as many as keep the grid within one CTA per SM
+    p.split = 4 * nblocks <= tr->sms ? 4 : (2 * nblocks <= tr->sms ? 2 : 1);
     p.pairs = (const float2 *)pairs;
     p.n_pairs = n;
     p.explicit_rows = explicit_rows;
@@ -612,7 +669,7 @@ su2_status trainer_launch(su2_trainer *tr, const float *pairs, long long n, int 
     p.k1 = (uint32_t)(tr->seed >> 32);
     p.partials = tr->partials;
     p.err = tr->err;
-    SU2_CUDA(launch_dependent(train::train_step_kernel, nblocks, train::kTrainThreads, sizeof(train::Smem), tr->stream,
+    SU2_CUDA(launch_dependent(train::train_step_kernel, nblocks * p.split, train::kTrainThreads, sizeof(train::Smem), tr->stream,
                               p));
     float bias1 = 1.0f, bias2 = 1.0f;
     if (lr > 0.0f) {
@@ -622,7 +679,7 @@ su2_status trainer_launch(su2_trainer *tr, const float *pairs, long long n, int 
     }
     SU2_CUDA(launch_dependent(train::adam_kernel, (train::kGradSlots + 63) / 64, 64, 0, tr->stream, tr->w, tr->m, tr->v,
                               (const float *)tr->partials, nblocks, 1.0f / (float)batch, lr, 0.9f, 0.999f, 1e-8f, bias1,
-                              bias2, tr->grad, loss_dst));
+                              bias2, tr->grad, loss_dst, tr->images));
     return SU2_OK;
 }
 
@@ -662,7 +719,7 @@ su2_status su2_trainer_create(const float *init_weights, uint64_t seed, void *cu
     tr->seed = seed;
     tr->partial_blocks = kMaxBatch / train::kRows;
     const size_t wb = 2048 * sizeof(float);
-    tr->block_bytes = 5 * wb + 256 + sizeof(float) * (size_t)tr->partial_blocks * train::kGradSlots;
+    tr->block_bytes = 5 * wb + 256 + train::kImageBytes + sizeof(float) * (size_t)tr->partial_blocks * train::kGradSlots;
     tr->block = device_alloc(tr->block_bytes, dev, tr->stream);
     if (!tr->block) {
         delete tr;
@@ -675,11 +732,17 @@ su2_status su2_trainer_create(const float *init_weights, uint64_t seed, void *cu
     tr->grad = (float *)(q + 3 * wb);
     tr->loss = (float *)(q + 4 * wb);
     tr->err = (unsigned int *)(q + 5 * wb);
-    tr->partials = (float *)(q + 5 * wb + 256);
+    tr->images = (unsigned char *)(q + 5 * wb + 256);
+    tr->partials = (float *)(q + 5 * wb + 256 + train::kImageBytes);
     su2_status st = SU2_OK;
-    cudaError_t e = cudaMemsetAsync(tr->block, 0, 5 * wb + 256, tr->stream);
+    cudaError_t e = cudaDeviceGetAttribute(&tr->sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaMemsetAsync(tr->block, 0, 5 * wb + 256 + train::kImageBytes, tr->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(tr->w, init_weights, sizeof(float) * learned::kWeights, cudaMemcpyHostToDevice, tr->stream);
+    if (e == cudaSuccess) {
+        train::put_images_kernel<<<(learned::kTrainable + 255) / 256, 256, 0, tr->stream>>>(tr->w, tr->images);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(tr->stream);
     if (e != cudaSuccess) st = cuda_fail(e, "su2_trainer_create");
     if (st != SU2_OK) {
@@ -706,9 +769,7 @@ su2_status su2_trainer_set_input_scaling(su2_trainer *tr, const float *dev_pairs
     if (!tr || !dev_pairs || n < 2) return SU2_E_INVAL;
     DeviceGuard guard(tr->device);
     // the block sums take the head of the step partials, idle between calls
-    int sms = 152;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, tr->device);
-    const int grid = (int)std::min<size_t>((n + 2047) / 2048, (size_t)sms);
+    const int grid = (int)std::min<size_t>((n + 2047) / 2048, (size_t)tr->sms);
     train::input_scaling_kernel<<<grid, train::kScalingThreads, 0, tr->stream>>>(
         (const float2 *)dev_pairs, (long long)n, (double *)tr->partials, tr->err + 16, tr->w);
     SU2_CUDA(cudaGetLastError());

@@ -1,5 +1,5 @@
 """The training kernels at the edges of their work split: one to 512 blocks of
-128 samples, and pair counts around the scaling kernel's 2048 pairs per block."""
+128 samples (four, two and one CTA per block), and pair counts around the scaling kernel's 2048 pairs per block."""
 import numpy as np
 import pytest
 
@@ -20,7 +20,7 @@ def _trainer(seed):
     return su2.su2_trainer_create(w, 1)
 
 
-@pytest.mark.parametrize("blocks", [1, 2, 33, 512])
+@pytest.mark.parametrize("blocks", [1, 38, 39, 76, 77, 512])
 def test_gradient_is_the_mean_of_its_blocks(blocks):
     """Rows of a block are summed in order and blocks in order, in binary32:
     the mean over n blocks differs from the binary64 mean of the blocks' own
