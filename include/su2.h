@@ -266,9 +266,13 @@ su2_status su2_set_timing(su2_lattice *lat, int enable);
  *   Creutz trial variable x = e + r1 (1 - e), r1 the log uniform of w,
  *   y2[i] = that trial's candidate a0 (Sec. 2), with e = exp(-2 beta k) as
  *   the heat-bath kernels set it up.  y2 may be NULL unless which is 2, 4, 5
- *   or 6. */
+ *   or 6.
+ * su2_selftest_rounding: n pairs (x, b); y[i] = 1/x (op 0), sqrt(x) (1),
+ *   sqrt(x) for x in [0, 1] (2) or x/b (3) as the draws compute it on operands
+ *   of known range, want[i] the same by the correctly rounded operation. */
 su2_status su2_selftest_philox(const uint32_t *ck, uint32_t *out, size_t n);
 su2_status su2_selftest_math(int which, const float *x, float *y, float *y2, size_t n);
+su2_status su2_selftest_rounding(int op, const float *xb, float *y, float *want, size_t n);
 
 /* ---------------------------------------------------------------------------
  * Learned proposal (not in the paper).  A small network of beta k (MLP

@@ -258,19 +258,22 @@ __device__ void batch_phase(const BatchParams &bp, int parity, uint32_t sweep, C
         }
 #pragma unroll 1
         for (int r = 0; r < rounds; ++r) {
+            const bool more = r + 1 < rounds;  // else: no next round to load
             const bool valid = cur <= last;
             const int nxt = cur + 32;
-            const int en = min(nxt, last);  // the last round reloads its own links: harmless
+            const int en = min(nxt, last);
             const Coord xn = eo_to_coord(g, en, parity);
             const int en_p = eo_fwd<MU>(g, xn, en);
             // ---- part 0
-            NuLinks nl = load_nu_eo<MU, OtherDir<MU, 0>::value, false>(links, g, xn, en, en_p, parity);
+            NuLinks nl = {};
+            if (more) nl = load_nu_eo<MU, OtherDir<MU, 0>::value, false>(links, g, xn, en, en_p, parity);
             const DrawSetup ds = prepare_draw(v_cur, beta);
             const uint4 w = philox_key(make_uint4((uint32_t)cur, sweep, sw_creutz, 0u), k0, k1);
-            float4 v_next = add_nu_terms(make_float4(0.0f, 0.0f, 0.0f, 0.0f), nl);
+            float4 v_next = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (more) v_next = add_nu_terms(v_next, nl);
             float4 sp_next = v_next;
             // ---- part 1
-            nl = load_nu_eo<MU, OtherDir<MU, 1>::value, false>(links, g, xn, en, en_p, parity);
+            if (more) nl = load_nu_eo<MU, OtherDir<MU, 1>::value, false>(links, g, xn, en, en_p, parity);
             {
                 bool first_ok;
                 float val;
@@ -280,12 +283,12 @@ __device__ void batch_phase(const BatchParams &bp, int parity, uint32_t sweep, C
                 push_done(ok, ds.ut, val, ds.ibk, cur, sp_cur);
                 push_retry(valid && !acc, ds.ut, ds.ibk, ds.e, cur, 1, sp_cur);
             }
-            v_next = add_nu_terms(v_next, nl);
+            if (more) v_next = add_nu_terms(v_next, nl);
             if (MU == 2) sp_next = v_next;
             // ---- part 2
-            nl = load_nu_eo<MU, OtherDir<MU, 2>::value, false>(links, g, xn, en, en_p, parity);
+            if (more) nl = load_nu_eo<MU, OtherDir<MU, 2>::value, false>(links, g, xn, en, en_p, parity);
             flush_done();
-            v_next = add_nu_terms(v_next, nl);
+            if (more) v_next = add_nu_terms(v_next, nl);
             if (MU == 3) sp_next = v_next;
             while (retry_n >= 32) {
                 retry_n -= 32;

@@ -18,9 +18,9 @@ namespace su2 {
 // staple is loaded one nu-group per stage while the current round is drawn
 // (part 0: k, U~^dag, the first trial's and the direction's Philox blocks;
 // part 1: the first trial; part 2: direction and store of accepted links).
-// A link whose first trial is rejected, or with beta k < 2 (then drawn by
-// Creutz's method, its staple queued in place of U~^dag), waits in the warp's
-// queue; 32 waiting links are finished together, and the queue is emptied at
+// A link whose first trial is rejected, or whose beta k is outside the main
+// path's range (kp_min_bk, kKpMaxBk; its staple queued in place of U~^dag,
+// below 2 drawn by Creutz's method), waits in the warp's queue; 32 waiting links are finished together, and the queue is emptied at
 // the segment's end.  MEAS: the segment's (1/2) Tr U'S sum goes to the slot
 // of its first chunk, as in batch_phase.
 template <int MU, int R, bool MEAS>
@@ -52,6 +52,7 @@ __device__ void batch_phase_kp(const BatchParams &bp, int parity, uint32_t sweep
         float4 *const links = sd.links;
         const uint32_t k0 = sd.k0, k1 = sd.k1;
         const float beta = sd.beta;
+        const float min_bk = kp_min_bk(beta);
         const int base0 = (chunk - lat_c0) * C;
         const int last = min((seg_end - lat_c0) * C, g.vh) - 1;
         const int rounds = (last - base0 + 32) >> 5;
@@ -64,12 +65,23 @@ __device__ void batch_phase_kp(const BatchParams &bp, int parity, uint32_t sweep
         auto retry = [&](int first, int n) {
             if (lane < n) {
                 const int q = first + lane;
-                const float4 ut = Q.r_ut[q];
-                const float bk_q = Q.r_ibk[q];
+                float4 ut = Q.r_ut[q];
+                float bk_q = Q.r_ibk[q];
                 const int eo = Q.r_eo[q];
                 float a0 = 0.0f;
                 int t = 1;
-                if (!(bk_q >= kKpMinBk)) {  // the queue holds the staple
+                if (!(bk_q >= min_bk && bk_q <= kKpMaxBk)) {
+                    // no trial yet, the queue holds the staple: checked operations
+                    const float4 v = ut;
+                    const float k = __fsqrt_rn(qnorm2(v));
+                    bk_q = __fmul_rn(beta, k);
+                    const float inv_k = __frcp_rn(k);
+                    if (bk_q >= kKpMinBk)
+                        ut = make_float4(__fmul_rn(v.x, inv_k), __fmul_rn(-v.y, inv_k), __fmul_rn(-v.z, inv_k),
+                                         __fmul_rn(-v.w, inv_k));
+                    t = 0;
+                }
+                if (!(bk_q >= kKpMinBk)) {  // Creutz's method
                     float4 out;
                     const int nt = heatbath_draw_gen(ut, beta, gen, (uint32_t)eo, sweep, (uint32_t)parity, MU, out);
                     if (nt > 0) {
@@ -120,17 +132,19 @@ __device__ void batch_phase_kp(const BatchParams &bp, int parity, uint32_t sweep
         uint4 dblk = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll 1
         for (int r = 0; r < rounds; ++r) {
+            const bool more = r + 1 < rounds;  // else: no next round to load
             const bool valid = cur <= last;
             const bool even_round = (r & 1) == 0;
             const int nxt = cur + 32;
-            const int en = min(nxt, last);  // the last round reloads its own links: harmless
+            const int en = min(nxt, last);
             const Coord xn = eo_to_coord(g, en, parity);
             const int en_p = eo_fwd<MU>(g, xn, en);
             // ---- part 0
-            NuLinks nl = load_nu_eo<MU, OtherDir<MU, 0>::value, false>(links, g, xn, en, en_p, parity);
+            NuLinks nl = {};
+            if (more) nl = load_nu_eo<MU, OtherDir<MU, 0>::value, false>(links, g, xn, en, en_p, parity);
             const float k = __fsqrt_rn(qnorm2(v_cur));
             const float bk = __fmul_rn(beta, k);
-            const bool use_kp = bk >= kKpMinBk;
+            const bool use_kp = bk >= min_bk && bk <= kKpMaxBk;
             const float inv_k = __frcp_rn(k);
             const float4 ut = make_float4(__fmul_rn(v_cur.x, inv_k), __fmul_rn(-v_cur.y, inv_k),
                                           __fmul_rn(-v_cur.z, inv_k), __fmul_rn(-v_cur.w, inv_k));
@@ -142,12 +156,13 @@ __device__ void batch_phase_kp(const BatchParams &bp, int parity, uint32_t sweep
             } else {
                 w = gen(w);
             }
-            float4 v_next = add_nu_terms(make_float4(0.0f, 0.0f, 0.0f, 0.0f), nl);
+            float4 v_next = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (more) v_next = add_nu_terms(v_next, nl);
             float4 sp_next = v_next;
             // ---- part 1
-            nl = load_nu_eo<MU, OtherDir<MU, 1>::value, false>(links, g, xn, en, en_p, parity);
+            if (more) nl = load_nu_eo<MU, OtherDir<MU, 1>::value, false>(links, g, xn, en, en_p, parity);
             float a0;
-            const bool first_ok = kp_trial(w, __fmul_rn(2.0f, bk), a0);
+            const bool first_ok = kp_trial<true>(w, __fmul_rn(2.0f, bk), a0);
             const bool accepted = valid && use_kp && first_ok;
             const bool park = valid && !(use_kp && first_ok);
             const unsigned int parked = __ballot_sync(0xffffffffu, park);
@@ -159,10 +174,10 @@ __device__ void batch_phase_kp(const BatchParams &bp, int parity, uint32_t sweep
                 if (MEAS) Q.r_sp[q] = sp_cur;
             }
             queued += __popc(parked);
-            v_next = add_nu_terms(v_next, nl);
+            if (more) v_next = add_nu_terms(v_next, nl);
             if (MU == 2) sp_next = v_next;
             // ---- part 2
-            nl = load_nu_eo<MU, OtherDir<MU, 2>::value, false>(links, g, xn, en, en_p, parity);
+            if (more) nl = load_nu_eo<MU, OtherDir<MU, 2>::value, false>(links, g, xn, en, en_p, parity);
             const int src = (even_round ? 0 : 16) + (lane >> 1);
             const uint4 wd = make_uint4(__shfl_sync(0xffffffffu, dblk.x, src), __shfl_sync(0xffffffffu, dblk.y, src),
                                         __shfl_sync(0xffffffffu, dblk.z, src), __shfl_sync(0xffffffffu, dblk.w, src));
@@ -170,7 +185,7 @@ __device__ void batch_phase_kp(const BatchParams &bp, int parity, uint32_t sweep
             if (accepted) links[link_index(g, MU, parity, cur)] = out;
             if (MEAS && accepted) plaq = __fadd_rn(plaq, qmul_re(out, sp_cur));
             my_trials += accepted ? 1u : 0u;
-            v_next = add_nu_terms(v_next, nl);
+            if (more) v_next = add_nu_terms(v_next, nl);
             if (MU == 3) sp_next = v_next;
             __syncwarp();
             if (queued >= 32) {

@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 
 #include "creutz_queue.cuh"
 #include "observables.cuh"
@@ -73,7 +74,18 @@ constexpr int kCrMinBlocks = SU2_HB_MIN_BLOCKS;  // blocks per SM the register b
 // of the plaquettes of planes (nu, MU) at x and x - nu, so over the odd sites
 // every such plaquette of the final configuration is counted once; the block
 // partial goes to p.plaq[block].
-template <int MU, bool MEAS, bool SLAB>
+//
+// PEEL: a warp's last round runs without loads of a next one.  Otherwise it
+// loads clamped links that nobody uses and waits for them, which is a round
+// trip to memory at the end of every launch; but the loop body is then in the
+// code twice, and at many rounds per warp the compiler's schedule of the pair
+// is the slower one.  us per phase with and without, measured every sweep,
+// beta = 4: 20^4 14.3 / 15.7, 24^4 17.9 / 19.4, 32^4 30.8 / 32.0, 36^4 (7.2
+// rounds) 44.8 / 45.5, 40^4 (11) 61.3 / 61.5, 44^4 83.8 / 83.2, 48^4 (22.7)
+// 113.6 / 111.8; so up to kCrPeelRounds.
+constexpr int kCrPeelRounds = 10;
+
+template <int MU, bool MEAS, bool SLAB, bool PEEL>
 __global__ void __launch_bounds__(kCrThreads, kCrMinBlocks) hb_phase_kernel(const HbParams p)
 {
     // a time slab updates its interior eo range; its random numbers are those
@@ -193,20 +205,23 @@ __global__ void __launch_bounds__(kCrThreads, kCrMinBlocks) hb_phase_kernel(cons
         v_cur = add_nu_terms(v_cur, load_nu_bases<MU, OtherDir<MU, 2>::value>(p.same, p.other, p.g, x, e, e_p));
         if (MU == 3) sp_cur = v_cur;
     }
-    while (base < eo_end) {  // warp-uniform
+    auto round = [&](auto more) {
+        constexpr bool MORE = decltype(more)::value;
         const bool valid = cur <= last;
         const int nxt = cur + stride;
         const int en = min(nxt, last);
         const Coord xn = eo_to_coord(p.g, en, p.parity);
         const int en_p = eo_fwd<MU>(p.g, xn, en);
         // ---- part 0
-        NuLinks nl = load_nu_bases<MU, OtherDir<MU, 0>::value>(p.same, p.other, p.g, xn, en, en_p);
+        NuLinks nl;
+        if constexpr (MORE) nl = load_nu_bases<MU, OtherDir<MU, 0>::value>(p.same, p.other, p.g, xn, en, en_p);
         const DrawSetup d = prepare_draw(v_cur, p.beta);
         const uint4 w = philox_rk(make_uint4((uint32_t)cur + rng_eo, sweep, sw_creutz, 0u), p.rk);
-        float4 v_next = add_nu_terms(make_float4(0.0f, 0.0f, 0.0f, 0.0f), nl);
+        float4 v_next = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if constexpr (MORE) v_next = add_nu_terms(v_next, nl);
         float4 sp_next = v_next;
         // ---- part 1
-        nl = load_nu_bases<MU, OtherDir<MU, 1>::value>(p.same, p.other, p.g, xn, en, en_p);
+        if constexpr (MORE) nl = load_nu_bases<MU, OtherDir<MU, 1>::value>(p.same, p.other, p.g, xn, en, en_p);
         {
             bool first_ok;
             float val;
@@ -216,12 +231,12 @@ __global__ void __launch_bounds__(kCrThreads, kCrMinBlocks) hb_phase_kernel(cons
             push_done(ok, d.ut, val, d.ibk, cur, sp_cur);
             push_retry(valid && !acc, d.ut, d.ibk, d.e, cur, 1, sp_cur);
         }
-        v_next = add_nu_terms(v_next, nl);
+        if constexpr (MORE) v_next = add_nu_terms(v_next, nl);
         if (MU == 2) sp_next = v_next;
         // ---- part 2
-        nl = load_nu_bases<MU, OtherDir<MU, 2>::value>(p.same, p.other, p.g, xn, en, en_p);
+        if constexpr (MORE) nl = load_nu_bases<MU, OtherDir<MU, 2>::value>(p.same, p.other, p.g, xn, en, en_p);
         flush_done();
-        v_next = add_nu_terms(v_next, nl);
+        if constexpr (MORE) v_next = add_nu_terms(v_next, nl);
         if (MU == 3) sp_next = v_next;
         while (retry_n >= 32) {
             retry_n -= 32;
@@ -231,6 +246,14 @@ __global__ void __launch_bounds__(kCrThreads, kCrMinBlocks) hb_phase_kernel(cons
         cur = nxt;
         v_cur = v_next;
         sp_cur = sp_next;
+    };
+    if (PEEL) {
+        if (base < eo_end) {  // warp-uniform
+            while (base + stride < eo_end) round(std::true_type{});
+            round(std::false_type{});
+        }
+    } else {
+        while (base < eo_end) round(std::true_type{});
     }
     while (retry_n > 0) {
         const int n = min(retry_n, 32);
@@ -249,7 +272,7 @@ __global__ void __launch_bounds__(kCrThreads, kCrMinBlocks) hb_phase_kernel(cons
     }
 }
 
-template <int MU, bool MEAS, bool SLAB = false>
+template <int MU, bool MEAS, bool SLAB = false, bool PEEL = true>
 static cudaError_t launch_hb(const HbParams &p, int device, cudaStream_t stream)
 {
     static int blocks_per_sm[64] = {};
@@ -257,7 +280,7 @@ static cudaError_t launch_hb(const HbParams &p, int device, cudaStream_t stream)
     if (device < 0 || device >= 64) device = 0;
     if (!blocks_per_sm[device]) {
         cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm[device],
-                                                                      hb_phase_kernel<MU, MEAS, SLAB>, kCrThreads, 0);
+                                                                      hb_phase_kernel<MU, MEAS, SLAB, PEEL>, kCrThreads, 0);
         if (e != cudaSuccess) return e;
         e = cudaDeviceGetAttribute(&num_sms[device], cudaDevAttrMultiProcessorCount, device);
         if (e != cudaSuccess) return e;
@@ -266,7 +289,8 @@ static cudaError_t launch_hb(const HbParams &p, int device, cudaStream_t stream)
     const int n = SLAB ? p.slab.eo_end - p.slab.eo_begin : p.g.vh;
     const int want = (n + kCrThreads - 1) / kCrThreads;
     const int grid = std::max(1, std::min(std::min(want, blocks_per_sm[device] * num_sms[device]), kFusedSlots));
-    hb_phase_kernel<MU, MEAS, SLAB><<<grid, kCrThreads, 0, stream>>>(p);
+    if (PEEL && n > kCrPeelRounds * grid * kCrThreads) return launch_hb<MU, MEAS, SLAB, false>(p, device, stream);
+    hb_phase_kernel<MU, MEAS, SLAB, PEEL><<<grid, kCrThreads, 0, stream>>>(p);
     return cudaGetLastError();
 }
 

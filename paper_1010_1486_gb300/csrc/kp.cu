@@ -9,6 +9,7 @@
 // accepts iff u <= 1 and r4^2 <= 1 - u (block t of the KP stream).  Links with
 // beta k < 2 are drawn by Creutz's method exactly as the plain kernel does.
 #include <algorithm>
+#include <type_traits>
 
 #include "kp_device.cuh"
 #include "observables.cuh"
@@ -30,6 +31,7 @@ struct KpParams {
     RoundKeys rk;
     int parity;
     float beta;
+    float min_bk;  // kp_min_bk(beta)
     uint32_t sweep;
     const uint32_t *sweep_dev;  // if non-NULL the sweep counter is read here (graph replays)
     int max_trials;             // trials a link may use before it keeps its old value
@@ -56,10 +58,12 @@ constexpr int kRetryCap = 64;  // per warp: at most 31 left over + 32 pushed by 
 //   part 1  the first trial;
 //   part 2  the direction and the store of every accepted link.
 // A link whose first trial is rejected is parked in the warp's retry queue
-// in shared memory (U~^dag, beta k, index), and so is a link with beta k < 2
-// (its staple in place of U~^dag), which the retry pass draws by Creutz's
-// method exactly as the plain kernel does; keeping that rare draw out of the
-// main loop leaves its registers to the pipeline (no spills).  Once 32 links wait, the whole
+// in shared memory (U~^dag, beta k, index), and so is a link whose beta k is
+// outside the range of the main path's operations (kp_min_bk, kKpMaxBk; its
+// staple in place of U~^dag): below 2 the retry pass draws it by Creutz's
+// method exactly as the plain kernel does.  Keeping that draw and every
+// range-checked operation out of the main loop leaves its registers to the
+// pipeline (no spills).  Once 32 links wait, the whole
 // warp runs their further trials 1, 2, ... together, so no warp spins on one
 // lane's rejections.  Every draw depends only on the link's counters, so the
 // phase computes exactly the one-thread-per-link definition.  Lanes past the
@@ -97,13 +101,24 @@ __global__ void __launch_bounds__(kKpThreads, kKpMinBlocks) kp_phase_kernel(cons
     auto retry = [&](int first, int n) {
         if (lane < n) {
             const int q = first + lane;
-            const float4 ut = s_ut[wib][q];
-            const float bk_q = s_bk[wib][q];
-            const float two_bk = __fmul_rn(2.0f, bk_q);
+            float4 ut = s_ut[wib][q];
+            float bk_q = s_bk[wib][q];
             const int eo = s_eo[wib][q];
             float a0 = 0.0f;
             int t = 1;
-            if (!(bk_q >= kKpMinBk)) {  // beta k < 2: Creutz's method; the queue holds the staple
+            if (!(bk_q >= p.min_bk && bk_q <= kKpMaxBk)) {
+                // no trial yet, the queue holds the staple: checked operations
+                const float4 v = ut;
+                const float k = __fsqrt_rn(qnorm2(v));
+                bk_q = __fmul_rn(p.beta, k);
+                const float inv_k = __frcp_rn(k);
+                if (bk_q >= kKpMinBk)
+                    ut = make_float4(__fmul_rn(v.x, inv_k), __fmul_rn(-v.y, inv_k), __fmul_rn(-v.z, inv_k),
+                                     __fmul_rn(-v.w, inv_k));
+                t = 0;
+            }
+            const float two_bk = __fmul_rn(2.0f, bk_q);
+            if (!(bk_q >= kKpMinBk)) {  // Creutz's method
                 float4 out;
                 const int n = heatbath_draw(ut, p.beta, p.rk, (uint32_t)eo + rng_eo, sweep, rng_parity, MU, out);
                 if (n > 0) {
@@ -160,17 +175,26 @@ __global__ void __launch_bounds__(kKpThreads, kKpMinBlocks) kp_phase_kernel(cons
     // words from the lane that drew its pair's block.
     bool even_round = true;
     uint4 dblk = make_uint4(0u, 0u, 0u, 0u);
-    while (base < eo_end) {  // warp-uniform
+    // A round; MORE: with the loads and the staple of the next one.  The last
+    // round of a warp runs without them (it used to load clamped links and wait
+    // for them: 24^4 at beta = 2.5 9.5 -> 8.0 us per phase, 8^4 4.3 -> 3.6,
+    // 48^4 70.5 -> 69.6).  Rounds that load keep the range-checked quotient in
+    // their logarithms: its branch keeps the compiler from moving the use of
+    // the loads forward (48^4: 71.4 us without it); the last has no loads to
+    // cover and takes the shorter form.
+    auto round = [&](auto more) {
+        constexpr bool MORE = decltype(more)::value;
         const bool valid = cur <= last;
         const int nxt = cur + stride;
         const int en = min(nxt, last);
         const Coord xn = eo_to_coord(p.g, en, p.parity);
         const int en_p = eo_fwd<MU>(p.g, xn, en);
         // ---- part 0
-        NuLinks nl = load_nu_bases<MU, OtherDir<MU, 0>::value>(p.same, p.other, p.g, xn, en, en_p);
+        NuLinks nl;
+        if constexpr (MORE) nl = load_nu_bases<MU, OtherDir<MU, 0>::value>(p.same, p.other, p.g, xn, en, en_p);
         const float k = __fsqrt_rn(qnorm2(v_cur));
         const float bk = __fmul_rn(p.beta, k);
-        const bool use_kp = bk >= kKpMinBk;
+        const bool use_kp = bk >= p.min_bk && bk <= kKpMaxBk;
         const float inv_k = __frcp_rn(k);
         const float4 ut = make_float4(__fmul_rn(v_cur.x, inv_k), __fmul_rn(-v_cur.y, inv_k),
                                       __fmul_rn(-v_cur.z, inv_k), __fmul_rn(-v_cur.w, inv_k));
@@ -182,14 +206,15 @@ __global__ void __launch_bounds__(kKpThreads, kKpMinBlocks) kp_phase_kernel(cons
         } else {
             w = philox_rk(w, p.rk);
         }
-        float4 v_next = add_nu_terms(make_float4(0.0f, 0.0f, 0.0f, 0.0f), nl);
+        float4 v_next = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if constexpr (MORE) v_next = add_nu_terms(v_next, nl);
         float4 sp_next = v_next;
         // ---- part 1
-        nl = load_nu_bases<MU, OtherDir<MU, 1>::value>(p.same, p.other, p.g, xn, en, en_p);
+        if constexpr (MORE) nl = load_nu_bases<MU, OtherDir<MU, 1>::value>(p.same, p.other, p.g, xn, en, en_p);
         float a0;
-        const bool first_ok = kp_trial(w, __fmul_rn(2.0f, bk), a0);
+        const bool first_ok = kp_trial<true, MORE>(w, __fmul_rn(2.0f, bk), a0);
         const bool accepted = valid && use_kp && first_ok;
-        const bool park = valid && !(use_kp && first_ok);  // rejected, or beta k < 2 (Creutz, in the queue)
+        const bool park = valid && !(use_kp && first_ok);  // rejected, or not drawn here
         const unsigned int parked = __ballot_sync(0xffffffffu, park);
         if (park) {  // rare at large beta k: a branch costs less than stores from every lane
             const int q = queued + __popc(parked & lanes_below);
@@ -199,10 +224,10 @@ __global__ void __launch_bounds__(kKpThreads, kKpMinBlocks) kp_phase_kernel(cons
             if (MEAS) s_sp[MEAS ? wib : 0][q] = sp_cur;
         }
         queued += __popc(parked);
-        v_next = add_nu_terms(v_next, nl);
+        if constexpr (MORE) v_next = add_nu_terms(v_next, nl);
         if (MU == 2) sp_next = v_next;
         // ---- part 2
-        nl = load_nu_bases<MU, OtherDir<MU, 2>::value>(p.same, p.other, p.g, xn, en, en_p);
+        if constexpr (MORE) nl = load_nu_bases<MU, OtherDir<MU, 2>::value>(p.same, p.other, p.g, xn, en, en_p);
         const int src = (even_round ? 0 : 16) + (lane >> 1);
         const uint4 wd = make_uint4(__shfl_sync(0xffffffffu, dblk.x, src), __shfl_sync(0xffffffffu, dblk.y, src),
                                     __shfl_sync(0xffffffffu, dblk.z, src), __shfl_sync(0xffffffffu, dblk.w, src));
@@ -210,7 +235,7 @@ __global__ void __launch_bounds__(kKpThreads, kKpMinBlocks) kp_phase_kernel(cons
         if (accepted) p.links[link_index(p.g, MU, p.parity, cur)] = out;
         if (MEAS && accepted) plaq = __fadd_rn(plaq, qmul_re(out, sp_cur));
         trials += accepted ? 1u : 0u;
-        v_next = add_nu_terms(v_next, nl);
+        if constexpr (MORE) v_next = add_nu_terms(v_next, nl);
         if (MU == 3) sp_next = v_next;
         __syncwarp();
         if (queued >= 32) {
@@ -222,6 +247,10 @@ __global__ void __launch_bounds__(kKpThreads, kKpMinBlocks) kp_phase_kernel(cons
         v_cur = v_next;
         sp_cur = sp_next;
         even_round = !even_round;
+    };
+    if (base < eo_end) {  // warp-uniform
+        while (base + stride < eo_end) round(std::true_type{});
+        round(std::false_type{});
     }
     if (queued > 0) retry(0, queued);
     const unsigned int wsum = __reduce_add_sync(0xffffffffu, trials);
@@ -263,6 +292,7 @@ su2_status launch_kp_phase(su2_lattice *lat, int mu, int parity, uint32_t sweep,
     p.rk = make_round_keys(lat->seed);
     p.parity = parity;
     p.beta = (float)lat->beta;
+    p.min_bk = kp_min_bk(p.beta);
     p.sweep = sweep;
     p.sweep_dev = lat->capturing ? lat->d_ctr : nullptr;
     p.max_trials = lat->max_trials;
@@ -298,6 +328,7 @@ su2_status launch_kp_phase_slab(su2_lattice *lat, int mu, int parity_local, uint
     p.rk = make_round_keys(lat->seed);
     p.parity = parity_local;
     p.beta = (float)lat->beta;
+    p.min_bk = kp_min_bk(p.beta);
     p.sweep = sweep;
     p.sweep_dev = nullptr;
     p.max_trials = lat->max_trials;

@@ -13,16 +13,29 @@
 namespace su2 {
 
 constexpr float kKpMinBk = 2.0f;
+// A link whose beta k lies in [lo, hi] is drawn with the range-limited
+// operations: hi = 2^60, and lo = 2 or, for beta above 2^31, beta 2^-30, so
+// that k (of the staple norm's square root) is within sqrt_in_range too.
+// Others take the checked operations, in the retry queue.
+constexpr float kKpMaxBk = 0x1p60f;
+__host__ __device__ inline float kp_min_bk(float beta)
+{
+    const float lo = beta * 0x1p-30f;
+    return lo > kKpMinBk ? lo : kKpMinBk;
+}
 constexpr uint32_t kKennedyPendleton = 5u;  // stream kind of the trials
 
 // One trial (block t of the KP stream): a0 = 1 - 2 u, and whether it is
-// accepted.
+// accepted.  IN_RANGE: 2 beta k is within the range of div_in_range (the
+// numerator is 0 or above 2^-80: |ln| >= 2^-24 unless zero, cos^2 >= 2^-43).
+template <bool IN_RANGE = false, bool CHECKED_LOG = false>
 __device__ __forceinline__ bool kp_trial(uint4 w, float two_bk, float &a0)
 {
     float sn, cs;
     sincos_2pi(uniform01(w.y), sn, cs);
-    const float num = __fmaf_rn(__fmul_rn(cs, cs), log_series(uniform_log(w.z)), log_series(uniform_log(w.x)));
-    const float lam2 = __fdiv_rn(-num, two_bk);
+    const float num = __fmaf_rn(__fmul_rn(cs, cs), log_series<CHECKED_LOG>(uniform_log(w.z)),
+                                log_series<CHECKED_LOG>(uniform_log(w.x)));
+    const float lam2 = IN_RANGE ? div_in_range(-num, two_bk) : __fdiv_rn(-num, two_bk);
     const float r4 = uniform01(w.w);
     a0 = __fmaf_rn(-2.0f, lam2, 1.0f);
     return lam2 <= 1.0f && __fmul_rn(r4, r4) <= __fsub_rn(1.0f, lam2);

@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "learned.cuh"
 #include "observables.cuh"
@@ -165,38 +166,47 @@ __global__ void __launch_bounds__(kLearnThreads, kLearnMinBlocks) learned_phase_
     __syncthreads();
     if (!s_table_ok) return;  // block-uniform
     tc::mbar_wait(&s_bar, 0, kTableWaitPolls);
-    while (base < p.g.vh) {  // warp-uniform
+    // a round; MORE: with the loads and the staple of the next one (the last
+    // round of a warp runs without them)
+    auto round = [&](auto more) {
+        constexpr bool MORE = decltype(more)::value;
         const bool valid = cur <= last;
         const int nxt = cur + stride;
         const int en = min(nxt, last);
         const Coord xn = eo_to_coord(p.g, en, p.parity);
         const int en_p = eo_fwd<MU>(p.g, xn, en);
         // ---- part 0
-        NuLinks nl = load_nu_bases<MU, OtherDir<MU, 0>::value>(p.same, p.other, p.g, xn, en, en_p);
+        NuLinks nl;
+        if constexpr (MORE) nl = load_nu_bases<MU, OtherDir<MU, 0>::value>(p.same, p.other, p.g, xn, en, en_p);
         const uint32_t li = link_index(p.g, MU, p.parity, min(cur, last));
         const float4 old = p.links[li];
         const uint4 w = philox_rk(make_uint4((uint32_t)cur, sweep, sw, 0u), p.rk);
         const learned::LearnedDraw r = learned::learned_propose(pr, p.beta, v_cur, uniform01(w.x));
-        float4 v_next = add_nu_terms(make_float4(0.0f, 0.0f, 0.0f, 0.0f), nl);
+        float4 v_next = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if constexpr (MORE) v_next = add_nu_terms(v_next, nl);
         float4 sp_next = v_next;
         // ---- part 1
-        nl = load_nu_bases<MU, OtherDir<MU, 1>::value>(p.same, p.other, p.g, xn, en, en_p);
+        if constexpr (MORE) nl = load_nu_bases<MU, OtherDir<MU, 1>::value>(p.same, p.other, p.g, xn, en, en_p);
         const bool ok = learned::learned_accept(r, old, uniform01(w.y), valid);
         const bool accept = valid && ok;
-        v_next = add_nu_terms(v_next, nl);
+        if constexpr (MORE) v_next = add_nu_terms(v_next, nl);
         if (MU == 2) sp_next = v_next;
         // ---- part 2
-        nl = load_nu_bases<MU, OtherDir<MU, 2>::value>(p.same, p.other, p.g, xn, en, en_p);
+        if constexpr (MORE) nl = load_nu_bases<MU, OtherDir<MU, 2>::value>(p.same, p.other, p.g, xn, en, en_p);
         const float4 out = direction_from_uniforms(r.a_new, r.d.ut, uniform01(w.z), uniform01(w.w));
         if (accept) p.links[li] = out;
         if (MEAS && valid) plaq = __fadd_rn(plaq, qmul_re(accept ? out : old, sp_cur));
         acc += accept ? 1u : 0u;
-        v_next = add_nu_terms(v_next, nl);
+        if constexpr (MORE) v_next = add_nu_terms(v_next, nl);
         if (MU == 3) sp_next = v_next;
         base += stride;
         cur = nxt;
         v_cur = v_next;
         sp_cur = sp_next;
+    };
+    if (base < p.g.vh) {  // warp-uniform
+        while (base + stride < p.g.vh) round(std::true_type{});
+        round(std::false_type{});
     }
     const unsigned int total = block_sum_u32(acc);
     if (threadIdx.x == 0 && total) {

@@ -5,6 +5,7 @@
 // the phase reads the staple (as the heat bath) plus the old link and writes
 // the new one, 144 bytes per link update.
 #include <algorithm>
+#include <type_traits>
 
 #include "observables.cuh"
 #include "staple.cuh"
@@ -31,9 +32,15 @@ struct OrParams {
 // U~^dag from the staple (identity if k = 0), as the heat bath's setup.
 __device__ __forceinline__ float4 staple_direction(float4 v)
 {
-    const float k = __fsqrt_rn(qnorm2(v));
-    if (!(k > 0.0f)) return make_float4(1.0f, 0.0f, 0.0f, 0.0f);
-    const float inv_k = __frcp_rn(k);
+    const float n2 = qnorm2(v);
+    float inv_k;
+    if (n2 >= 0x1p-70f && n2 <= 0x1p100f) {
+        inv_k = rcp_in_range(sqrt_in_range(n2));
+    } else {
+        const float k = __fsqrt_rn(n2);
+        if (!(k > 0.0f)) return make_float4(1.0f, 0.0f, 0.0f, 0.0f);
+        inv_k = __frcp_rn(k);
+    }
     return make_float4(__fmul_rn(v.x, inv_k), __fmul_rn(-v.y, inv_k), __fmul_rn(-v.z, inv_k),
                        __fmul_rn(-v.w, inv_k));
 }
@@ -47,7 +54,15 @@ __device__ __forceinline__ float4 staple_direction(float4 v)
 // results, so the loop body has no divergent branch.  MEAS: the plaquette
 // contributions (1/2) Tr U'S, S the staple terms of nu < MU, as in the
 // heat-bath kernels.
-template <int MU, bool MEAS>
+//
+// PEEL: a warp's last round runs without loads of a next one, as in the
+// heat-bath kernel.  us per phase with and without, beta = 4: 20^4 5.1 / 6.2,
+// 24^4 6.2 / 8.2, 28^4 8.2 / 10.2, 32^4 (3.4 rounds) 12.0 / 12.3, 36^4 (5.4)
+// 22.8 / 22.9, 40^4 (8.2) 32.4 / 31.6, 48^4 (17) 62.2 / 61.0; so up to
+// kOrPeelRounds.
+constexpr int kOrPeelRounds = 6;
+
+template <int MU, bool MEAS, bool PEEL>
 __global__ void __launch_bounds__(kOrThreads, kOrMinBlocks) or_phase_kernel(const OrParams p)
 {
     const int stride = gridDim.x * kOrThreads;
@@ -68,35 +83,46 @@ __global__ void __launch_bounds__(kOrThreads, kOrMinBlocks) or_phase_kernel(cons
         v_cur = add_nu_terms(v_cur, load_nu_bases<MU, OtherDir<MU, 2>::value>(p.same, p.other, p.g, x, e, e_p));
         if (MU == 3) sp_cur = v_cur;
     }
-    while (base < p.g.vh) {  // warp-uniform
+    auto round = [&](auto more) {
+        constexpr bool MORE = decltype(more)::value;
         const bool valid = cur <= last;
         const int nxt = cur + stride;
         const int en = min(nxt, last);
         const Coord xn = eo_to_coord(p.g, en, p.parity);
         const int en_p = eo_fwd<MU>(p.g, xn, en);
         // ---- part 0
-        NuLinks nl = load_nu_bases<MU, OtherDir<MU, 0>::value>(p.same, p.other, p.g, xn, en, en_p);
+        NuLinks nl;
+        if constexpr (MORE) nl = load_nu_bases<MU, OtherDir<MU, 0>::value>(p.same, p.other, p.g, xn, en, en_p);
         const uint32_t li = link_index(p.g, MU, p.parity, min(cur, last));
         const float4 old = p.links[li];
         const float4 ut = staple_direction(v_cur);
-        float4 v_next = add_nu_terms(make_float4(0.0f, 0.0f, 0.0f, 0.0f), nl);
+        float4 v_next = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if constexpr (MORE) v_next = add_nu_terms(v_next, nl);
         float4 sp_next = v_next;
         // ---- part 1
-        nl = load_nu_bases<MU, OtherDir<MU, 1>::value>(p.same, p.other, p.g, xn, en, en_p);
+        if constexpr (MORE) nl = load_nu_bases<MU, OtherDir<MU, 1>::value>(p.same, p.other, p.g, xn, en, en_p);
         const float4 t = qmul(ut, qdag(old));
-        v_next = add_nu_terms(v_next, nl);
+        if constexpr (MORE) v_next = add_nu_terms(v_next, nl);
         if (MU == 2) sp_next = v_next;
         // ---- part 2
-        nl = load_nu_bases<MU, OtherDir<MU, 2>::value>(p.same, p.other, p.g, xn, en, en_p);
+        if constexpr (MORE) nl = load_nu_bases<MU, OtherDir<MU, 2>::value>(p.same, p.other, p.g, xn, en, en_p);
         const float4 out = qmul(t, ut);
         if (valid) p.links[li] = out;
         if (MEAS && valid) plaq = __fadd_rn(plaq, qmul_re(out, sp_cur));
-        v_next = add_nu_terms(v_next, nl);
+        if constexpr (MORE) v_next = add_nu_terms(v_next, nl);
         if (MU == 3) sp_next = v_next;
         base += stride;
         cur = nxt;
         v_cur = v_next;
         sp_cur = sp_next;
+    };
+    if (PEEL) {
+        if (base < p.g.vh) {  // warp-uniform
+            while (base + stride < p.g.vh) round(std::true_type{});
+            round(std::false_type{});
+        }
+    } else {
+        while (base < p.g.vh) round(std::true_type{});
     }
     if (MEAS) {
         const double total = block_sum((double)plaq);
@@ -104,22 +130,23 @@ __global__ void __launch_bounds__(kOrThreads, kOrMinBlocks) or_phase_kernel(cons
     }
 }
 
-template <int MU, bool MEAS>
+template <int MU, bool MEAS, bool PEEL = true>
 static cudaError_t launch_or(const OrParams &p, int device, cudaStream_t stream)
 {
     static int per_sm[64] = {};
     static int sms[64] = {};
     if (device < 0 || device >= 64) device = 0;
     if (!per_sm[device]) {
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[device], or_phase_kernel<MU, MEAS>,
-                                                                      kOrThreads, 0);
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[device],
+                                                                      or_phase_kernel<MU, MEAS, PEEL>, kOrThreads, 0);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms[device], cudaDevAttrMultiProcessorCount, device);
         if (e != cudaSuccess) return e;
         per_sm[device] = std::max(1, per_sm[device]);
     }
     const int want = (p.g.vh + kOrThreads - 1) / kOrThreads;
     const int grid = std::max(1, std::min(std::min(want, per_sm[device] * sms[device]), kFusedSlots));
-    or_phase_kernel<MU, MEAS><<<grid, kOrThreads, 0, stream>>>(p);
+    if (PEEL && p.g.vh > kOrPeelRounds * grid * kOrThreads) return launch_or<MU, MEAS, false>(p, device, stream);
+    or_phase_kernel<MU, MEAS, PEEL><<<grid, kOrThreads, 0, stream>>>(p);
     return cudaGetLastError();
 }
 

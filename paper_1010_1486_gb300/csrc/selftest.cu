@@ -61,6 +61,18 @@ __global__ void math_selftest_kernel(int which, const float *__restrict__ x, flo
     }
 }
 
+// op 0: 1/x, 1: sqrt(x), 2: sqrt(x) on [0, 1], 3: x/b, by the range-limited
+// operations (y) and by the checked ones (want).
+__global__ void rounding_selftest_kernel(int op, const float2 *__restrict__ xb, float *__restrict__ y,
+                                         float *__restrict__ want, size_t n)
+{
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const float x = xb[i].x, b = xb[i].y;
+        y[i] = op == 0 ? rcp_in_range(x) : op == 1 ? sqrt_in_range(x) : op == 2 ? sqrt_unit(x) : div_in_range(x, b);
+        want[i] = op == 0 ? __frcp_rn(x) : op == 3 ? __fdiv_rn(x, b) : __fsqrt_rn(x);
+    }
+}
+
 // Copies host input to a temporary device buffer, runs `launch`, copies back.
 template <typename Launch>
 static su2_status run_with_buffers(const void *in, size_t in_bytes, void *out, size_t out_bytes, void *out2,
@@ -120,6 +132,16 @@ su2_status su2_selftest_math(int which, const float *x, float *y, float *y2, siz
                                 math_selftest_kernel<<<grid_for((int64_t)n, 256), 256, 0, s>>>(
                                     which, (const float *)in, (float *)o, (float *)o2, n);
                             });
+}
+
+su2_status su2_selftest_rounding(int op, const float *xb, float *y, float *want, size_t n)
+{
+    if (!xb || !y || !want || op < 0 || op > 3) return SU2_E_INVAL;
+    if (n == 0) return SU2_OK;
+    return run_with_buffers(xb, 8 * n, y, 4 * n, want, 4 * n, [op, n](char *in, char *o, char *o2, cudaStream_t s) {
+        rounding_selftest_kernel<<<grid_for((int64_t)n, 256), 256, 0, s>>>(op, (const float2 *)in, (float *)o,
+                                                                           (float *)o2, n);
+    });
 }
 
 }  // extern "C"

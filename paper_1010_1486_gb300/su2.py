@@ -107,6 +107,7 @@ _SIGS = {
     "su2_set_overrelax": [_P, _i32],
     "su2_selftest_philox": [_P, _P, ctypes.c_size_t],
     "su2_selftest_math": [_i32, _P, _P, _P, ctypes.c_size_t],
+    "su2_selftest_rounding": [_i32, _P, _P, _P, ctypes.c_size_t],
     "su2_plaquette_noalloc": [_P, _i32, _i32, _P, _P],
     "su2_batch_create": [_i32, _P, _P, _P, _P, _i32, _P, ctypes.POINTER(_P)],
     "su2_batch_destroy": [_P],
@@ -407,6 +408,19 @@ def su2_selftest_math(which: int, x: np.ndarray):
         y = y.reshape(x.shape)
         y2 = y2.reshape(x.shape) if y2 is not None else None
     return (y, y2) if y2 is not None else y
+
+
+def su2_selftest_rounding(op: int, x: np.ndarray, b: np.ndarray | None = None):
+    """(range-limited, correctly rounded) results of op 0: 1/x, 1: sqrt(x),
+    2: sqrt(x) on [0, 1], 3: x/b."""
+    xb = np.zeros((x.size, 2), dtype=np.float32)
+    xb[:, 0] = x
+    if b is not None:
+        xb[:, 1] = b
+    y, want = np.empty(x.size, dtype=np.float32), np.empty(x.size, dtype=np.float32)
+    _check(_lib.su2_selftest_rounding(op, _host_ptr(xb), _host_ptr(y), _host_ptr(want), x.size),
+           "su2_selftest_rounding")
+    return y, want
 
 
 def su2_plaquette_noalloc(links_ptr: int, ns: int, nt: int, out_ptr: int, stream=None) -> None:
