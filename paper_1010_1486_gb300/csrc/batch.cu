@@ -171,8 +171,13 @@ cudaError_t enqueue_launch(su2_batch *b, int do_sweep, int measure)
     if (e != cudaSuccess) return e;
     BatchParams p = params_of(b, do_sweep, measure);
     void *args[] = {&p};
-    return cudaLaunchCooperativeKernel(kernel_for(b->sampler, b->R, b->threads), dim3(b->grid), dim3(b->threads),
-                                       args, 0,
+    // no more blocks than have work (a warp per chunk and per measurement
+    // round): the others would only lengthen the grid barriers
+    const int items = std::max(do_sweep ? b->total_chunks : 0,
+                               measure ? (do_sweep ? b->total_poly_rounds : b->total_mrounds) : 0);
+    const int warps = b->threads / 32;
+    const int grid = std::max(1, std::min(b->grid, (items + warps - 1) / warps));
+    return cudaLaunchCooperativeKernel(kernel_for(b->sampler, b->R, b->threads), dim3(grid), dim3(b->threads), args, 0,
                                        b->stream);
 }
 

@@ -30,12 +30,15 @@ struct LatDesc {
     int npoly_rounds;  // ceil(Ns^3 / 32) rounds of Polyakov lines
 };
 
+// Arrivals and release on lines of their own: the polls of the waiting blocks
+// do not slow the atomics of the arriving ones.  Zeroed before every launch;
+// both numbers only grow during it.
 struct BarrierState {
-    unsigned int count;
-    unsigned int gen;
-    unsigned int error;  // bit 0: a barrier wait timed out
-    unsigned int pad;
+    alignas(128) unsigned int count;  // arrivals
+    alignas(128) unsigned int gen;    // barriers completed
+    unsigned int error;               // bit 0: a barrier wait timed out
 };
+static_assert(sizeof(BarrierState) == 256, "the barrier self-test places its counter behind it");
 
 struct BatchParams {
     const LatDesc *desc;        // [n]
@@ -70,37 +73,40 @@ __device__ __forceinline__ unsigned long long global_time_ns()
     return t;
 }
 
-// Grid-wide barrier for a cooperative launch (all blocks co-resident).  Every
-// wait is bounded by timeout_ns: on expiry the block sets bar->error and all
-// blocks stop waiting; the function then returns false everywhere and the
-// caller abandons the sweep.
-static __device__ bool grid_barrier(BarrierState *bar, unsigned long long timeout_ns)
+// Grid-wide barrier number `passed` (0, 1, ...) of a cooperative launch (all
+// blocks co-resident).  Arrival is one release-acquire atomic per block, and
+// the waits poll with acquire loads; the clock is read every kBarrierPolls
+// polls only.  Every wait is bounded by timeout_ns: on expiry the block sets
+// bar->error and releases the others; the function then returns false
+// everywhere and the caller abandons the sweep.  (With both numbers on one
+// line, a clock read and 100 ns of sleep per poll, and all co-resident blocks
+// taking part: nine uneven lattices 192 -> 124 us per measured sweep, 64 of
+// them 464 -> 460.)
+constexpr int kBarrierPolls = 64;
+
+static __device__ bool grid_barrier(BarrierState *bar, unsigned int passed, unsigned long long timeout_ns)
 {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        volatile unsigned int *vgen = &bar->gen;
-        volatile unsigned int *verr = &bar->error;
-        const unsigned int g = *vgen;
-        __threadfence();
-        const unsigned int arrived = atomicAdd(&bar->count, 1u) + 1u;
-        if (arrived == gridDim.x) {
-            atomicExch(&bar->count, 0u);
-            __threadfence();
-            atomicAdd(&bar->gen, 1u);
+        unsigned int before, gen = 0u;
+        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(before) : "l"(&bar->count) : "memory");
+        if (before + 1u == gridDim.x * (passed + 1u)) {
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&bar->gen), "r"(passed + 1u) : "memory");
         } else {
             const unsigned long long t0 = global_time_ns();
-            while (*vgen == g) {
-                if (*verr & 1u) break;
-                if (global_time_ns() - t0 > timeout_ns) {
+            for (int polls = 1;; ++polls) {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(gen) : "l"(&bar->gen) : "memory");
+                if (gen > passed) break;
+                if (polls % kBarrierPolls == 0 && global_time_ns() - t0 > timeout_ns) {
                     atomicOr(&bar->error, 1u);
+                    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&bar->gen), "r"(0xffffffffu) : "memory");
                     break;
                 }
-                __nanosleep(100);
+                __nanosleep(40);
             }
         }
-        __threadfence();
-        ok = (*verr & 1u) == 0u;
+        ok = (*(volatile unsigned int *)&bar->error & 1u) == 0u;
     }
     __syncthreads();
     return ok != 0;
@@ -415,6 +421,7 @@ __global__ void __launch_bounds__(T, kBatchThreadsPerSm / T) batch_sweep_kernel(
     const unsigned int slot = *(volatile unsigned int *)bp.meas_index;
     const bool fused = bp.fused && (int)slot < bp.history_cap;
     bool ok = true;
+    unsigned int barriers = 0;
     if (bp.do_sweep) {
         for (int ph = 0; ph < 8 && ok; ++ph) {
             const int parity = ph & 1;
@@ -439,12 +446,12 @@ __global__ void __launch_bounds__(T, kBatchThreadsPerSm / T) batch_sweep_kernel(
             if (lane == 0 && wsum)
                 atomicAdd(&bp.trial_slots[ph * kTrialSlots + (warp_global & (kTrialSlots - 1))],
                           (unsigned long long)wsum);
-            ok = grid_barrier(bp.bar, bp.timeout_ns);
+            ok = grid_barrier(bp.bar, barriers++, bp.timeout_ns);
         }
     }
     if (ok && bp.measure && (int)slot < bp.history_cap) {
         batch_measure_rounds(bp);
-        ok = grid_barrier(bp.bar, bp.timeout_ns);
+        ok = grid_barrier(bp.bar, barriers++, bp.timeout_ns);
         if (ok) batch_measure_final(bp, slot);
     }
     if (ok && blockIdx.x == 0 && threadIdx.x == 0) {
