@@ -597,14 +597,18 @@ static su2_status generate_enqueue(su2_lattice *lat, int nsweeps, int measure_ev
     }
     lat->hb_log.used = 0;
     lat->or_log.used = 0;
+    bool done = false;
+    if (small_lattice(lat) && (st = small_sweeps(lat, nsweeps, measure_every, reunit_every, lat->scratch.history,
+                                                 lat->scratch.history + lat->scratch.history_cap, &done)) != SU2_OK)
+        return st;
     // Graph replays need a stream that can be captured and no per-launch events.
-    bool graphs = lat->stream != nullptr && !lat->timing && !lat->graphs_off && nsweeps >= 1;
+    bool graphs = !done && lat->stream != nullptr && !lat->timing && !lat->graphs_off && nsweeps >= 1;
     if (graphs) {
         set_counters_kernel<<<1, 1, 0, lat->stream>>>(lat->d_ctr, lat->sweep);
         SU2_CUDA(cudaGetLastError());
     }
     int m = 0;
-    for (int s = 1; s <= nsweeps; ++s) {
+    for (int s = 1; s <= nsweeps && !done; ++s) {
         const bool measure = measure_every > 0 && s % measure_every == 0;
         const bool reunit = reunit_every > 0 && s % reunit_every == 0;
         if (graphs) {
@@ -672,7 +676,9 @@ su2_status su2_heatbath_sweep(su2_lattice *lat, int nsweeps, su2_stats *stats)
     su2_status st;
     lat->hb_log.used = 0;
     lat->or_log.used = 0;
-    for (int s = 0; s < nsweeps; ++s)
+    bool done = false;
+    if (small_lattice(lat) && (st = small_sweeps(lat, nsweeps, 0, 0, nullptr, nullptr, &done)) != SU2_OK) return st;
+    for (int s = 0; s < nsweeps && !done; ++s)
         if ((st = one_sweep(lat)) != SU2_OK) return st;
     lat->hb_log.used = 0;
     lat->or_log.used = 0;

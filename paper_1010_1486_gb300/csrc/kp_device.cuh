@@ -25,20 +25,33 @@ __host__ __device__ inline float kp_min_bk(float beta)
 }
 constexpr uint32_t kKennedyPendleton = 5u;  // stream kind of the trials
 
-// One trial (block t of the KP stream): a0 = 1 - 2 u, and whether it is
-// accepted.  IN_RANGE: 2 beta k is within the range of div_in_range (the
-// numerator is 0 or above 2^-80: |ln| >= 2^-24 unless zero, cos^2 >= 2^-43).
-template <bool IN_RANGE = false, bool CHECKED_LOG = false>
-__device__ __forceinline__ bool kp_trial(uint4 w, float two_bk, float &a0)
+// The part of a trial that does not need the staple: cos^2(2 pi r2) ln r3 + ln r1.
+template <bool CHECKED_LOG = false>
+__device__ __forceinline__ float kp_numerator(uint4 w)
 {
     float sn, cs;
     sincos_2pi(uniform01(w.y), sn, cs);
-    const float num = __fmaf_rn(__fmul_rn(cs, cs), log_series<CHECKED_LOG>(uniform_log(w.z)),
-                                log_series<CHECKED_LOG>(uniform_log(w.x)));
+    return __fmaf_rn(__fmul_rn(cs, cs), log_series<CHECKED_LOG>(uniform_log(w.z)),
+                     log_series<CHECKED_LOG>(uniform_log(w.x)));
+}
+
+// ... and the rest: a0 = 1 - 2 u, and whether it is accepted.
+template <bool IN_RANGE>
+__device__ __forceinline__ bool kp_candidate(float num, uint32_t w3, float two_bk, float &a0)
+{
     const float lam2 = IN_RANGE ? div_in_range(-num, two_bk) : __fdiv_rn(-num, two_bk);
-    const float r4 = uniform01(w.w);
+    const float r4 = uniform01(w3);
     a0 = __fmaf_rn(-2.0f, lam2, 1.0f);
     return lam2 <= 1.0f && __fmul_rn(r4, r4) <= __fsub_rn(1.0f, lam2);
+}
+
+// One trial (block t of the KP stream).  IN_RANGE: 2 beta k is within the
+// range of div_in_range (the numerator is 0 or above 2^-80: |ln| >= 2^-24
+// unless zero, cos^2 >= 2^-43).
+template <bool IN_RANGE = false, bool CHECKED_LOG = false>
+__device__ __forceinline__ bool kp_trial(uint4 w, float two_bk, float &a0)
+{
+    return kp_candidate<IN_RANGE>(kp_numerator<CHECKED_LOG>(w), w.w, two_bk, a0);
 }
 
 }  // namespace su2

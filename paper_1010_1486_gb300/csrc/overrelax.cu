@@ -29,22 +29,6 @@ struct OrParams {
     const float4 *other[4];  // ... at the opposite parity
 };
 
-// U~^dag from the staple (identity if k = 0), as the heat bath's setup.
-__device__ __forceinline__ float4 staple_direction(float4 v)
-{
-    const float n2 = qnorm2(v);
-    float inv_k;
-    if (n2 >= 0x1p-70f && n2 <= 0x1p100f) {
-        inv_k = rcp_in_range(sqrt_in_range(n2));
-    } else {
-        const float k = __fsqrt_rn(n2);
-        if (!(k > 0.0f)) return make_float4(1.0f, 0.0f, 0.0f, 0.0f);
-        inv_k = __frcp_rn(k);
-    }
-    return make_float4(__fmul_rn(v.x, inv_k), __fmul_rn(-v.y, inv_k), __fmul_rn(-v.z, inv_k),
-                       __fmul_rn(-v.w, inv_k));
-}
-
 // Persistent grid: warp w takes the rounds of 32 consecutive links w, w + W,
 // ... (W warps).  Each loop iteration (three per round) issues the six loads
 // of one nu-group of the next round, does one third of the current round's

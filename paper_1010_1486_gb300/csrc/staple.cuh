@@ -46,6 +46,22 @@ __device__ __forceinline__ float4 add_nu_terms(float4 v, const NuLinks &n)
     return qmul_add(qmul(qdag(n.nu_xpm), qdag(n.mu_xm)), n.nu_xm, v);
 }
 
+// U~^dag from the staple (identity if k = 0), as the heat bath's setup.
+__device__ __forceinline__ float4 staple_direction(float4 v)
+{
+    const float n2 = qnorm2(v);
+    float inv_k;
+    if (n2 >= 0x1p-70f && n2 <= 0x1p100f) {
+        inv_k = rcp_in_range(sqrt_in_range(n2));
+    } else {
+        const float k = __fsqrt_rn(n2);
+        if (!(k > 0.0f)) return make_float4(1.0f, 0.0f, 0.0f, 0.0f);
+        inv_k = __frcp_rn(k);
+    }
+    return make_float4(__fmul_rn(v.x, inv_k), __fmul_rn(-v.y, inv_k), __fmul_rn(-v.z, inv_k),
+                       __fmul_rn(-v.w, inv_k));
+}
+
 // Even/odd neighbour indices straight from the coordinates.  The strides of
 // y, z, t are even, so (lex +- stride) >> 1 = eo +- stride/2 (and the
 // periodic jump is even too); in x the step depends on the parity of x0.

@@ -80,6 +80,8 @@ struct su2_lattice {
     su2::GenGraph gen_graph[4];    // captured sweeps, variant = (measured) | (reunitarized) << 1
     su2::GenGraph learned_graph[2];  // captured learned sweeps, [measured]
 
+    int small_room[2] = {0, 0};  // per sampler: whether the one-launch sweeps fit the device (small_sweeps)
+
     bool timing = false;
     su2::EventLog hb_log;  // heat-bath (and learned) phase launches
     su2::EventLog or_log;  // over-relaxation phase launches
@@ -212,6 +214,13 @@ su2_status launch_kp_phase(su2_lattice *lat, int mu, int parity, uint32_t sweep,
 su2_status launch_hb_phase_slab(su2_lattice *lat, int mu, int parity_local, uint32_t sweep, const SlabRange &r);
 su2_status launch_kp_phase_slab(su2_lattice *lat, int mu, int parity_local, uint32_t sweep, const SlabRange &r);
 su2_status launch_reunitarize(su2_lattice *lat);
+// Sweeps of a small lattice in one launch (small.cu): whether the lattice is
+// one, and nsweeps sweeps with their over-relaxation, reunitarizations and
+// measurements (plaq, poly: device, one value per measured sweep), enqueued.
+// *done is false, and nothing enqueued, where the device has no room for them.
+bool small_lattice(const su2_lattice *lat);
+su2_status small_sweeps(su2_lattice *lat, int nsweeps, int measure_every, int reunit_every, double *plaq, double *poly,
+                        bool *done);
 // Observables: write the value into *dst (device memory) without synchronising.
 su2_status launch_plaquette(su2_lattice *lat, double *dst);
 su2_status launch_polyakov(su2_lattice *lat, double *dst);
