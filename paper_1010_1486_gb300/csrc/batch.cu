@@ -211,15 +211,22 @@ su2_status launch_sweep(su2_batch *b, int measure)
     return SU2_OK;
 }
 
-su2_status check_flags(su2_batch *b, su2_stats *stats, uint64_t sweeps, int launches)
+// Places in the block from the barrier state on.
+constexpr size_t kCountersAt = 256, kTrialsAt = 512;
+constexpr size_t kCheckBytes = kTrialsAt + sizeof(unsigned long long) * 8 * kTrialSlots;
+static_assert(sizeof(BarrierState) <= kCountersAt, "the counters follow the barrier state");
+
+// Reads the batch's status (synchronises), through the first kCheckBytes of `page` if it has one.
+su2_status check_flags(su2_batch *b, su2_stats *stats, uint64_t sweeps, int launches, const HostPage &page)
 {
-    unsigned long long slots[8 * kTrialSlots];
-    unsigned int counters[4];
-    BarrierState bar;
-    SU2_CUDA(cudaMemcpyAsync(slots, b->d_trials, sizeof slots, cudaMemcpyDeviceToHost, b->stream));
-    SU2_CUDA(cudaMemcpyAsync(counters, b->d_counters, sizeof counters, cudaMemcpyDeviceToHost, b->stream));
-    SU2_CUDA(cudaMemcpyAsync(&bar, b->d_bar, sizeof bar, cudaMemcpyDeviceToHost, b->stream));
+    // barrier state, counters and trial counters lie side by side: one copy
+    alignas(128) char own[kCheckBytes];
+    char *const to = page.p ? page.p : own;
+    SU2_CUDA(cudaMemcpyAsync(to, b->d_bar, kCheckBytes, cudaMemcpyDeviceToHost, b->stream));
     SU2_CUDA(cudaStreamSynchronize(b->stream));
+    const BarrierState &bar = *(const BarrierState *)to;
+    const unsigned int *const counters = (const unsigned int *)(to + kCountersAt);
+    const unsigned long long *const slots = (const unsigned long long *)(to + kTrialsAt);
     uint64_t sites = 0;
     for (const Geom &g : b->geom) sites += 2ull * (uint64_t)g.vh;
     if (stats) {
@@ -307,6 +314,7 @@ su2_status su2_batch_create(int n, const int *ns, const int *nt, const double *b
     }
     su2_batch *b = new (std::nothrow) su2_batch();
     if (!b) return SU2_E_NOMEM;
+    host_pages_retain();
     b->n = n;
     b->device = dev;
     b->stream = (cudaStream_t)cuda_stream;
@@ -345,14 +353,15 @@ su2_status su2_batch_create(int n, const int *ns, const int *nt, const double *b
     b->total_poly_rounds = (int)poly_rounds.size();
     const size_t owner_bytes = align256(sizeof(int) * max_chunks) + align256(sizeof(int) * b->total_mrounds) +
                                align256(sizeof(int2) * poly_rounds.size());
-    const size_t bar_bytes = align256(sizeof(BarrierState));
-    const size_t counter_bytes = align256(sizeof(unsigned int) * 8);
+    const size_t bar_bytes = kCountersAt;  // check_flags reads barrier state, counters and trials as one range
+    const size_t counter_bytes = kTrialsAt - kCountersAt;
     const size_t trial_bytes = align256(sizeof(unsigned long long) * 8 * kTrialSlots);
     b->block_bytes = links_bytes + desc_bytes + 2 * prefix_bytes + partial_bytes + chunk_bytes + owner_bytes +
                      bar_bytes + counter_bytes + trial_bytes;
     b->block = device_alloc(b->block_bytes, dev, b->stream);
     if (!b->block) {
         delete b;
+        host_pages_release();
         set_last_error("device allocation of the batch failed");
         return SU2_E_NOMEM;
     }
@@ -449,6 +458,7 @@ su2_status su2_batch_destroy(su2_batch *b)
     device_free(b->block, b->block_bytes, b->device, b->stream);
     const cudaError_t e = cudaStreamSynchronize(b->stream);
     delete b;
+    host_pages_release();
     if (e != cudaSuccess) return cuda_fail(e, "su2_batch_destroy");
     return SU2_OK;
 }
@@ -467,12 +477,18 @@ su2_status su2_batch_generate(su2_batch *b, int nsweeps, int measure_every, doub
         const int measure = (measure_every > 0 && s % measure_every == 0) ? 1 : 0;
         if ((st = launch_sweep(b, measure)) != SU2_OK) return st;
     }
-    st = check_flags(b, stats, (uint64_t)nsweeps, nsweeps);
-    if (nmeas > 0 && (plaq || poly)) {
-        std::vector<double> h((size_t)nmeas * 2 * b->n);
-        SU2_CUDA(cudaMemcpyAsync(h.data(), b->d_history, sizeof(double) * h.size(), cudaMemcpyDeviceToHost,
-                                 b->stream));
-        SU2_CUDA(cudaStreamSynchronize(b->stream));
+    const HostPage page;
+    const size_t values = nmeas > 0 && (plaq || poly) ? (size_t)nmeas * 2 * b->n : 0;
+    std::vector<double> own;
+    double *h = (double *)(page.p + kCheckBytes);
+    if (!page.p || kCheckBytes + sizeof(double) * values > kHostPageBytes) {
+        own.resize(values);
+        h = own.data();
+    }
+    if (values)
+        SU2_CUDA(cudaMemcpyAsync(h, b->d_history, sizeof(double) * values, cudaMemcpyDeviceToHost, b->stream));
+    st = check_flags(b, stats, (uint64_t)nsweeps, nsweeps, page);
+    if (values && st != SU2_E_CUDA) {
         for (int m = 0; m < nmeas; ++m)
             for (int l = 0; l < b->n; ++l) {
                 if (plaq) plaq[(size_t)m * b->n + l] = h[((size_t)m * 2 + 0) * b->n + l];

@@ -647,10 +647,16 @@ su2_status su2_generate(su2_lattice *lat, int nsweeps, int measure_every, int re
 {
     if (!lat || nsweeps < 0 || measure_every < 0 || reunit_every < 0) return SU2_E_INVAL;
     DeviceGuard guard(lat->device);
-    su2_status st = generate_enqueue(lat, nsweeps, measure_every, reunit_every, plaq, poly, true);
-    if (st != SU2_OK) return st;
+    const HostPage page;
+    ResultCopy copy(page, kStatsBytes, measure_every > 0 ? nsweeps / measure_every : 0, plaq, poly);
+    su2_status st = generate_enqueue(lat, nsweeps, measure_every, reunit_every, copy.plaq, copy.poly, true);
+    if (st != SU2_OK) {
+        cudaStreamSynchronize(lat->stream);  // nothing may still be on its way to the page
+        return st;
+    }
     if (stats) memset(stats, 0, sizeof *stats);
-    st = collect_stats(lat, stats, (uint64_t)nsweeps);
+    st = collect_stats(lat, stats, (uint64_t)nsweeps, page);
+    copy.finish();
     if (stats) {
         stats->kernel_launches = (uint32_t)(8 * nsweeps);
         stats->overrelax_sweeps = (uint64_t)nsweeps * (uint64_t)lat->overrelax;

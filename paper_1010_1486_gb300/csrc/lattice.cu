@@ -65,6 +65,49 @@ void device_free(void *ptr, size_t bytes, int device, cudaStream_t stream)
     cudaFreeAsync(ptr, stream);
 }
 
+// ------------------------------------------------- page-locked result pages
+static std::mutex g_page_mutex;
+static char *g_pages[kHostPages];  // the free ones
+static int g_pages_free = 0, g_pages_made = 0, g_page_users = 0;
+
+HostPage::HostPage() : p(nullptr)
+{
+    std::lock_guard<std::mutex> lock(g_page_mutex);
+    if (g_pages_free > 0) {
+        p = g_pages[--g_pages_free];
+    } else if (g_pages_made < kHostPages) {
+        void *q = nullptr;
+        if (cudaHostAlloc(&q, kHostPageBytes, cudaHostAllocPortable) == cudaSuccess) {
+            p = (char *)q;
+            ++g_pages_made;
+        } else {
+            cudaGetLastError();
+        }
+    }
+}
+
+HostPage::~HostPage()
+{
+    if (!p) return;
+    std::lock_guard<std::mutex> lock(g_page_mutex);
+    g_pages[g_pages_free++] = p;
+}
+
+void host_pages_retain()
+{
+    std::lock_guard<std::mutex> lock(g_page_mutex);
+    ++g_page_users;
+}
+
+void host_pages_release()
+{
+    std::lock_guard<std::mutex> lock(g_page_mutex);
+    if (--g_page_users > 0) return;
+    g_pages_made -= g_pages_free;
+    while (g_pages_free > 0) cudaFreeHost(g_pages[--g_pages_free]);
+    cudaGetLastError();
+}
+
 // ------------------------------------------------------------- kernels
 __global__ void cold_start_kernel(float4 *__restrict__ links, int64_t n)
 {
@@ -170,18 +213,19 @@ su2_status launch_reunitarize(su2_lattice *lat)
 
 su2_status launch_clear_counters(su2_lattice *lat)
 {
-    SU2_CUDA(cudaMemsetAsync(lat->scratch.trials, 0, sizeof(unsigned long long) * 8 * kTrialSlots, lat->stream));
-    SU2_CUDA(cudaMemsetAsync(lat->scratch.flags, 0, sizeof(unsigned int) * 4, lat->stream));
+    // the flags follow the trial counters
+    SU2_CUDA(cudaMemsetAsync(lat->scratch.trials, 0, kStatsBytes, lat->stream));
     return SU2_OK;
 }
 
-su2_status collect_stats(su2_lattice *lat, su2_stats *stats, uint64_t sweeps)
+su2_status collect_stats(su2_lattice *lat, su2_stats *stats, uint64_t sweeps, const HostPage &page)
 {
-    unsigned long long slots[8 * kTrialSlots];
-    unsigned int flags[4];
-    SU2_CUDA(cudaMemcpyAsync(slots, lat->scratch.trials, sizeof slots, cudaMemcpyDeviceToHost, lat->stream));
-    SU2_CUDA(cudaMemcpyAsync(flags, lat->scratch.flags, sizeof flags, cudaMemcpyDeviceToHost, lat->stream));
+    alignas(8) char own[kStatsBytes];
+    char *const to = page.p ? page.p : own;
+    SU2_CUDA(cudaMemcpyAsync(to, lat->scratch.trials, kStatsBytes, cudaMemcpyDeviceToHost, lat->stream));
     SU2_CUDA(cudaStreamSynchronize(lat->stream));
+    const unsigned long long *const slots = (const unsigned long long *)to;
+    const unsigned int *const flags = (const unsigned int *)(slots + 8 * kTrialSlots);
     if (stats) {
         for (int ph = 0; ph < 8; ++ph) {
             uint64_t s = 0;
@@ -312,6 +356,7 @@ su2_status su2_create(int ns, int nt, double beta, uint64_t seed, su2_start star
 
     su2_lattice *lat = new (std::nothrow) su2_lattice();
     if (!lat) return SU2_E_NOMEM;
+    host_pages_retain();
     lat->ns = ns;
     lat->nt = nt;
     lat->vol = (int64_t)ns * ns * ns * nt;
@@ -329,7 +374,7 @@ su2_status su2_create(int ns, int nt, double beta, uint64_t seed, su2_start star
     const size_t partials_bytes = align256(sizeof(double) * partials_cap);
     const size_t ticket_bytes = align256(sizeof(unsigned int) * 4);
     const size_t result_bytes = align256(sizeof(double) * 4);
-    const size_t trials_bytes = align256(sizeof(unsigned long long) * 8 * kTrialSlots);
+    const size_t trials_bytes = sizeof(unsigned long long) * 8 * kTrialSlots;  // the flags follow directly
     const size_t flags_bytes = align256(sizeof(unsigned int) * 4);
     const size_t ctr_bytes = align256(sizeof(uint32_t) * 2);
     lat->block_bytes =
@@ -337,6 +382,7 @@ su2_status su2_create(int ns, int nt, double beta, uint64_t seed, su2_start star
     lat->block = device_alloc(lat->block_bytes, dev, lat->stream);
     if (!lat->block) {
         delete lat;
+        host_pages_release();
         set_last_error("device allocation of the lattice failed");
         return SU2_E_NOMEM;
     }
@@ -396,6 +442,7 @@ su2_status su2_destroy(su2_lattice *lat)
     device_free(lat->block, lat->block_bytes, lat->device, lat->stream);
     cudaError_t e = cudaStreamSynchronize(lat->stream);
     delete lat;
+    host_pages_release();
     if (e != cudaSuccess) return cuda_fail(e, "su2_destroy");
     return SU2_OK;
 }
@@ -502,8 +549,10 @@ su2_status su2_sync(su2_lattice *lat)
 {
     if (!lat) return SU2_E_INVAL;
     DeviceGuard guard(lat->device);
-    unsigned int flags[4];
-    SU2_CUDA(cudaMemcpyAsync(flags, lat->scratch.flags, sizeof flags, cudaMemcpyDeviceToHost, lat->stream));
+    const HostPage page;
+    unsigned int own[4];
+    unsigned int *const flags = page.p ? (unsigned int *)page.p : own;
+    SU2_CUDA(cudaMemcpyAsync(flags, lat->scratch.flags, sizeof own, cudaMemcpyDeviceToHost, lat->stream));
     SU2_CUDA(cudaStreamSynchronize(lat->stream));
     if (flags[0] != 0) {
         SU2_CUDA(cudaMemsetAsync(lat->scratch.flags, 0, sizeof(unsigned int), lat->stream));
@@ -518,20 +567,16 @@ su2_status su2_check_links(su2_lattice *lat, double tol, uint64_t *nonfinite, ui
 {
     if (!lat || !(tol >= 0.0)) return SU2_E_INVAL;
     DeviceGuard guard(lat->device);
-    unsigned long long *d = (unsigned long long *)device_alloc(2 * sizeof(unsigned long long), lat->device,
-                                                               lat->stream);
-    if (!d) return SU2_E_NOMEM;
-    unsigned long long h[2] = {0ull, 0ull};
-    cudaError_t e = cudaMemsetAsync(d, 0, sizeof h, lat->stream);
-    if (e == cudaSuccess) {
-        check_links_kernel<<<grid_for(4 * lat->vol, 256, 152 * 8), 256, 0, lat->stream>>>(lat->links, 4 * lat->vol,
-                                                                                          (float)tol, d);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h, d, sizeof h, cudaMemcpyDeviceToHost, lat->stream);
-    device_free(d, 2 * sizeof(unsigned long long), lat->device, lat->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(lat->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "su2_check_links");
+    unsigned long long *const d = (unsigned long long *)(lat->scratch.result + 2);
+    const HostPage page;
+    unsigned long long own[2];
+    unsigned long long *const h = page.p ? (unsigned long long *)page.p : own;
+    SU2_CUDA(cudaMemsetAsync(d, 0, sizeof own, lat->stream));
+    check_links_kernel<<<grid_for(4 * lat->vol, 256, 152 * 8), 256, 0, lat->stream>>>(lat->links, 4 * lat->vol,
+                                                                                      (float)tol, d);
+    SU2_CUDA(cudaGetLastError());
+    SU2_CUDA(cudaMemcpyAsync(h, d, sizeof own, cudaMemcpyDeviceToHost, lat->stream));
+    SU2_CUDA(cudaStreamSynchronize(lat->stream));
     if (nonfinite) *nonfinite = h[0];
     if (off_norm) *off_norm = h[1];
     if (h[0]) {

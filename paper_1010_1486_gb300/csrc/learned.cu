@@ -580,19 +580,27 @@ su2_status su2_learned_generate(su2_lattice *lat, int nsweeps, int measure_every
         lat->sweep += 1;
         if (measure) ++m;
     }
+    // the trial counters, the acceptance counters and control words (one copy:
+    // they lie side by side), then the measurements
+    const HostPage page;
+    const size_t accept_at = kStatsBytes, accept_bytes = 256 + sizeof(unsigned long long) * 8 * kAcceptSlots;
+    alignas(8) char own[accept_bytes];
+    char *const to = page.p ? page.p + accept_at : own;
+    ResultCopy copy(page, accept_at + accept_bytes, nmeas, plaq, poly);
     if (nmeas > 0 && plaq)
-        SU2_CUDA(cudaMemcpyAsync(plaq, lat->scratch.history, sizeof(double) * nmeas, cudaMemcpyDeviceToHost,
+        SU2_CUDA(cudaMemcpyAsync(copy.plaq, lat->scratch.history, sizeof(double) * nmeas, cudaMemcpyDeviceToHost,
                                  lat->stream));
     if (nmeas > 0 && poly)
-        SU2_CUDA(cudaMemcpyAsync(poly, lat->scratch.history + lat->scratch.history_cap, sizeof(double) * nmeas,
+        SU2_CUDA(cudaMemcpyAsync(copy.poly, lat->scratch.history + lat->scratch.history_cap, sizeof(double) * nmeas,
                                  cudaMemcpyDeviceToHost, lat->stream));
-    unsigned long long slots[8 * kAcceptSlots];
-    unsigned int ctl[4];
-    SU2_CUDA(cudaMemcpyAsync(slots, lat->accept_slots, sizeof slots, cudaMemcpyDeviceToHost, lat->stream));
-    SU2_CUDA(cudaMemcpyAsync(ctl, lat->learned_ctl, sizeof ctl, cudaMemcpyDeviceToHost, lat->stream));
+    static_assert(sizeof(unsigned int) * 4 <= 256, "the control words' place before the acceptance counters");
+    SU2_CUDA(cudaMemcpyAsync(to, lat->learned_ctl, accept_bytes, cudaMemcpyDeviceToHost, lat->stream));
     su2_stats plain;
     memset(&plain, 0, sizeof plain);
-    st = collect_stats(lat, &plain, (uint64_t)nsweeps);
+    st = collect_stats(lat, &plain, (uint64_t)nsweeps, page);
+    copy.finish();
+    const unsigned int *const ctl = (const unsigned int *)to;
+    const unsigned long long *const slots = (const unsigned long long *)(to + 256);
     double kms = 0.0;
     su2_status st_t = timing_read(lat, lat->hb_log, &kms);
     if (st == SU2_OK) st = st_t;

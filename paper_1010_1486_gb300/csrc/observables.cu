@@ -197,28 +197,33 @@ su2_status fused_finish_with_polyakov(su2_lattice *lat, double *plaq_dst, double
 
 using namespace su2;
 
+// Runs an observable and brings its value to the host: the kernel writes it
+// into a page-locked page itself, or, when none is free, to *dev to be copied.
+static su2_status read_value(su2_lattice *lat, su2_status (*launch)(su2_lattice *, double *), double *dev, double *out)
+{
+    const HostPage page;
+    su2_status st = launch(lat, page.p ? (double *)page.p : dev);
+    if (st != SU2_OK) return st;
+    if (!page.p) SU2_CUDA(cudaMemcpyAsync(out, dev, sizeof(double), cudaMemcpyDeviceToHost, lat->stream));
+    SU2_CUDA(cudaStreamSynchronize(lat->stream));
+    if (page.p) *out = *(const double *)page.p;
+    return SU2_OK;
+}
+
 extern "C" {
 
 su2_status su2_plaquette(su2_lattice *lat, double *out)
 {
     if (!lat || !out) return SU2_E_INVAL;
     DeviceGuard guard(lat->device);
-    su2_status st = launch_plaquette(lat, lat->scratch.result);
-    if (st != SU2_OK) return st;
-    SU2_CUDA(cudaMemcpyAsync(out, lat->scratch.result, sizeof(double), cudaMemcpyDeviceToHost, lat->stream));
-    SU2_CUDA(cudaStreamSynchronize(lat->stream));
-    return SU2_OK;
+    return read_value(lat, launch_plaquette, lat->scratch.result, out);
 }
 
 su2_status su2_polyakov(su2_lattice *lat, double *out)
 {
     if (!lat || !out) return SU2_E_INVAL;
     DeviceGuard guard(lat->device);
-    su2_status st = launch_polyakov(lat, lat->scratch.result + 1);
-    if (st != SU2_OK) return st;
-    SU2_CUDA(cudaMemcpyAsync(out, lat->scratch.result + 1, sizeof(double), cudaMemcpyDeviceToHost, lat->stream));
-    SU2_CUDA(cudaStreamSynchronize(lat->stream));
-    return SU2_OK;
+    return read_value(lat, launch_polyakov, lat->scratch.result + 1, out);
 }
 
 }  // extern "C"

@@ -27,7 +27,7 @@ constexpr int kFusedRegion = 6 * kFusedSlots;
 struct DeviceScratch {
     double *partials = nullptr;             // per-block partial sums of a reduction
     unsigned int *ticket = nullptr;         // last-block counter of a reduction
-    double *result = nullptr;               // [0] plaquette, [1] Polyakov (latest)
+    double *result = nullptr;               // [0] plaquette, [1] Polyakov (latest), [2], [3] counts of su2_check_links
     unsigned long long *trials = nullptr;   // [8][kTrialSlots]
     unsigned int *flags = nullptr;          // [0] sampler cap hits, [1] other errors
     double *history = nullptr;              // measurements of su2_generate: [2][history_cap]
@@ -118,6 +118,51 @@ su2_status cuda_fail(cudaError_t e, const char *what);
         cudaError_t e_ = (call);                                               \
         if (e_ != cudaSuccess) return ::su2::cuda_fail(e_, #call);             \
     } while (0)
+
+// A page of page-locked host memory for the results of a synchronous call:
+// copies to it are queued behind the kernels, where a copy to pageable memory
+// waits for them (about 8 us each, one after the other).  Pages come from a
+// process-wide pool of at most kHostPages, taken for the duration of a call;
+// p is NULL when none is free (or page-locking failed), and the call then
+// copies to its caller's memory directly.
+constexpr size_t kHostPageBytes = 64 * 1024;
+constexpr int kHostPages = 16;
+struct HostPage {
+    char *p;
+    HostPage();
+    ~HostPage();
+    HostPage(const HostPage &) = delete;
+    HostPage &operator=(const HostPage &) = delete;
+};
+
+// Every lattice and batch retains the pages while it lives; the last one to go
+// gives them back.
+void host_pages_retain();
+void host_pages_release();
+
+// The two measurement histories of a call: their device copies go to plaq and
+// poly here -- behind the first `used` bytes of the page if they fit, else the
+// caller's arrays -- and finish(), after the synchronisation, hands them on.
+struct ResultCopy {
+    double *plaq, *poly;  // where to copy to (NULL where the caller wants none)
+    double *const user_plaq, *const user_poly;
+    const size_t n;
+    ResultCopy(const HostPage &page, size_t used, int nmeas, double *up, double *ul)
+        : plaq(up), poly(ul), user_plaq(up), user_poly(ul), n(nmeas > 0 ? (size_t)nmeas : 0)
+    {
+        if (!page.p || used + 2 * n * sizeof(double) > kHostPageBytes) return;
+        double *const at = (double *)(page.p + used);
+        if (up) plaq = at;
+        if (ul) poly = at + n;
+    }
+    void finish() const
+    {
+        for (size_t i = 0; i < n; ++i) {
+            if (plaq != user_plaq) user_plaq[i] = plaq[i];
+            if (poly != user_poly) user_poly[i] = poly[i];
+        }
+    }
+};
 
 // Keeps the lattice's device current for the duration of a call.
 struct DeviceGuard {
@@ -233,7 +278,9 @@ su2_status timing_read(su2_lattice *lat, EventLog &log, double *ms);
 // Over-relaxation: one phase, and `n` sweeps (8 phases each, timed into or_log).
 su2_status launch_or_phase(su2_lattice *lat, int mu, int parity);
 su2_status overrelax_sweeps(su2_lattice *lat, int n);
-// Reads and clears the trial counters and flags (synchronises).
-su2_status collect_stats(su2_lattice *lat, su2_stats *stats, uint64_t sweeps);
+// Reads the trial counters and flags (synchronises), through the first
+// kStatsBytes of `page` if it has one.
+constexpr size_t kStatsBytes = 8 * kTrialSlots * sizeof(unsigned long long) + 4 * sizeof(unsigned int);
+su2_status collect_stats(su2_lattice *lat, su2_stats *stats, uint64_t sweeps, const HostPage &page);
 
 }  // namespace su2

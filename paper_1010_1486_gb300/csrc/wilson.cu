@@ -456,7 +456,9 @@ extern "C" su2_status su2_wilson_loops(su2_lattice *lat, int rmax, int tmax, dou
     DeviceGuard guard(lat->device);
     const size_t n_out = (size_t)rmax * (size_t)tmax;
     const size_t bytes = sizeof(double) * n_out;
-    double host[kWilsonMaxR * kWilsonMaxT + 1];
+    const HostPage page;
+    double own[kWilsonMaxR * kWilsonMaxT + 1];
+    double *const host = page.p ? (double *)page.p : own;
     double *d_tiles = nullptr;
     SU2_CUDA(launch_tiles(lat, rmax, tmax, &d_tiles));
     SU2_CUDA(cudaMemcpyAsync(host, d_tiles, bytes + sizeof(double), cudaMemcpyDeviceToHost, lat->stream));
