@@ -14,25 +14,72 @@
 
 namespace su2 {
 
+// Mean plaquette.  A thread takes one spatial site and walks along t: the
+// links U_0..U_2 that it reads at t + 1 for the planes with t are its own links
+// of the next step, and the block's 384 consecutive pairs of sites (both
+// spatial parities, a warp for 32 pairs of one parity: every load is 512
+// contiguous bytes) find most of their neighbours in y in L1, where the block
+// itself read them.  Thirteen loads per site remain, all in flight at once.
+// One site per thread in lexicographic order (sixteen loads, two runs of 256
+// bytes each) was bound by L1 wavefronts (88%), and the same by even/odd order
+// by the traffic from L2 (87 us, 12.7 TB/s).  48^4: 100 -> 90 us per call, 82 us
+// (ncu) in the kernel, which waits for its loads (24 warps per SM, 78
+// registers); splitting the planes into two groups of loads, one in flight
+// while the other is computed, spills (102 us) or halves the warps (106 us).
+constexpr int kPlaqPairs = 384;                 // pairs of sites (2 j, 2 j + 1) per block
+constexpr int kPlaqThreads = 2 * kPlaqPairs;    // one block per SM
+
 // dst (+ *idx when idx is given: the measurement slot of a graph replay)
-__global__ void __launch_bounds__(kReduceThreads, 4) plaquette_kernel(const float4 *__restrict__ L, Geom g,
-                                                                   double *__restrict__ partials,
-                                                                   unsigned int *__restrict__ ticket,
-                                                                   double *__restrict__ dst,
-                                                                   const uint32_t *__restrict__ idx)
+__global__ void __launch_bounds__(kPlaqThreads, 1) plaquette_kernel(const float4 *__restrict__ L, Geom g, int pair_blocks,
+                                                                  int t_chunk, double *__restrict__ partials,
+                                                                  unsigned int *__restrict__ ticket,
+                                                                  double *__restrict__ dst,
+                                                                  const uint32_t *__restrict__ idx)
 {
-    float acc = 0.0f;  // per-thread partial in binary32; the block and grid sums are binary64
-    const int64_t vol = 2 * (int64_t)g.vh;
-    // sites in lexicographic order (both parities interleaved), so the
-    // neighbour links a block reads were just read by its neighbours (L2)
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < vol; s += (int64_t)gridDim.x * blockDim.x) {
-        const int eo = (int)(s >> 1);
-        const int parity = (int)(s & 1) ^ (eo_to_coord(g, eo, 0).lex != 2 * eo);
-        const Coord x = eo_to_coord(g, eo, parity);
-        acc = __fadd_rn(acc, site_plaquette(L, g, x, eo, parity));
+    double acc = 0.0;
+    const int half = g.vs >> 1;
+    const int chunk = (int)blockIdx.x / pair_blocks;
+    const int sp = (int)threadIdx.x >= kPlaqPairs;  // spatial parity, warp-uniform
+    const int j = ((int)blockIdx.x - chunk * pair_blocks) * kPlaqPairs + (int)threadIdx.x - sp * kPlaqPairs;
+    const int t0 = chunk * t_chunk, t1 = min(t0 + t_chunk, g.nt);
+    if (j < half && t0 < t1) {
+        const uint32_t r1 = fastdiv(2u * (uint32_t)j, g.div_ns), z = fastdiv(r1, g.div_ns);
+        const int y = (int)(r1 - z * (uint32_t)g.ns);
+        const int x = 2 * j - (int)r1 * g.ns + ((y + (int)z + sp) & 1);
+        // the pair indices of x + 0, x + 1, x + 2 (at the other parity)
+        const int f[3] = {j + (x & 1) - (x == g.ns - 1 ? g.ns >> 1 : 0),
+                          y == g.ns - 1 ? j - (g.wrap[1] >> 1) : j + (g.stride[1] >> 1),
+                          (int)z == g.ns - 1 ? j - (g.wrap[2] >> 1) : j + (g.stride[2] >> 1)};
+        float4 u[4];
+#pragma unroll
+        for (int mu = 0; mu < 3; ++mu) u[mu] = __ldg(L + link_index(g, mu, (sp + t0) & 1, t0 * half + j));
+#pragma unroll 1
+        for (int t = t0; t < t1; ++t) {
+            const int parity = (sp + t) & 1, op = parity ^ 1, at = t * half;
+            const int ahead = (t == g.nt - 1 ? 0 : at + half) + j;
+            float4 b[3][4], c[3];  // b[mu][nu] = U_nu(x + mu); U_mu(x + nu) for nu < 3 is b[nu][mu]; c[mu] = U_mu(x + t)
+            u[3] = __ldg(L + link_index(g, 3, parity, at + j));
+#pragma unroll
+            for (int mu = 0; mu < 3; ++mu) {
+                c[mu] = __ldg(L + link_index(g, mu, op, ahead));
+#pragma unroll
+                for (int nu = 0; nu < 4; ++nu)
+                    if (nu != mu) b[mu][nu] = __ldg(L + link_index(g, nu, op, at + f[mu]));
+            }
+            float sum = 0.0f;
+#pragma unroll
+            for (int mu = 0; mu < 3; ++mu)
+#pragma unroll
+                for (int nu = mu + 1; nu < 4; ++nu)
+                    sum = __fadd_rn(sum, qmul_re(qmul(qmul(u[mu], b[mu][nu]), qdag(nu == 3 ? c[mu] : b[nu][mu])),
+                                                 qdag(u[nu])));
+            acc += (double)sum;
+#pragma unroll
+            for (int mu = 0; mu < 3; ++mu) u[mu] = c[mu];
+        }
     }
-    const double total = block_sum((double)acc);
-    finish_reduction(total, partials, ticket, idx ? dst + *idx : dst, 1.0 / (6.0 * (double)vol));
+    const double total = block_sum(acc);
+    finish_reduction(total, partials, ticket, idx ? dst + *idx : dst, 1.0 / (12.0 * (double)g.vh));
 }
 
 // (1/2) Tr of U_3(x,0) U_3(x,1) ... U_3(x,Nt-1).  A block of kPolySeg warps
@@ -142,14 +189,16 @@ __global__ void __launch_bounds__(kPolyThreads) polyakov_kernel(const float4 *__
 su2_status launch_plaquette(su2_lattice *lat, double *dst)
 {
     const Geom g = geom_of(lat);
-    // persistent grid (4 blocks of 256 per SM): each thread sums several
-    // sites, one block reduction per block
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, lat->device);
-    const int grid = grid_for(lat->vol, kReduceThreads, std::min(lat->scratch.partials_cap, 4 * sms));
-    plaquette_kernel<<<grid, kReduceThreads, 0, lat->stream>>>(lat->links, g, lat->scratch.partials,
-                                                               lat->scratch.ticket, dst,
-                                                               lat->capturing ? lat->d_ctr + 1 : nullptr);
+    // one block per SM: the time extent in as many chunks as fill them
+    const int pair_blocks = (g.vs / 2 + kPlaqPairs - 1) / kPlaqPairs;
+    const int chunks = std::max(1, std::min(lat->nt, sms / pair_blocks));
+    const int t_chunk = (lat->nt + chunks - 1) / chunks;
+    const int grid = pair_blocks * ((lat->nt + t_chunk - 1) / t_chunk);
+    plaquette_kernel<<<grid, kPlaqThreads, 0, lat->stream>>>(lat->links, g, pair_blocks, t_chunk,
+                                                             lat->scratch.partials, lat->scratch.ticket, dst,
+                                                             lat->capturing ? lat->d_ctr + 1 : nullptr);
     SU2_CUDA(cudaGetLastError());
     return SU2_OK;
 }

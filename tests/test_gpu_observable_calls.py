@@ -1,12 +1,29 @@
-"""The page-locked result pages under more threads than there are pages."""
+"""The plaquette kernel's walk along t at the edges of its split, and the
+page-locked result pages under more threads than there are pages."""
 import threading
 
 import numpy as np
 import pytest
 
+import oracle
 from paper_1010_1486_gb300 import su2
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("ns,nt", [(2, 2), (2, 40), (4, 6), (10, 6), (10, 18), (28, 2), (28, 6), (36, 4), (56, 2)])
+def test_plaquette_is_the_mean_of_its_sites(ns, nt):
+    """Blocks of 384 pairs, ragged in space and time, one to many chunks of t:
+    the oracle's binary32 site values, summed in binary64 on both sides."""
+    h = su2.su2_create(ns, nt, 2.3, 5 + ns, su2.SU2_HOT)
+    try:
+        got = su2.su2_plaquette(h)
+        links = su2.su2_get_links(h, ns, nt)
+    finally:
+        su2.su2_destroy(h)
+    sites = oracle.site_plaquettes(ns, nt, links).astype(np.float64)
+    # |site| <= 6 over 6 V; N binary64 additions in another order
+    assert abs(got - sites.sum() / (6.0 * sites.size)) <= sites.size * 2.0 ** -53
 
 
 def test_many_threads_read_their_own_results():
