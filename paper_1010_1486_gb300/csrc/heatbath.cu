@@ -94,7 +94,10 @@ __global__ void __launch_bounds__(kCrThreads, kCrMinBlocks) hb_phase_kernel(cons
     const int eo_end = SLAB ? p.slab.eo_end : p.g.vh;
     const uint32_t rng_eo = SLAB ? p.slab.rng_eo : 0u;
     const uint32_t rng_parity = SLAB ? (uint32_t)p.slab.rng_parity : (uint32_t)p.parity;
-    if (p.gate != nullptr && *(volatile const unsigned int *)p.gate == 1u) return;
+    if (p.gate != nullptr && *(volatile const unsigned int *)p.gate == 1u) {
+        if (MEAS && threadIdx.x == 0) p.plaq[blockIdx.x] = 0.0;
+        return;
+    }
     __shared__ CrQueues s_q[kCrWarps];
     const uint32_t sweep = p.sweep_dev ? *p.sweep_dev : p.sweep;
     const int lane = threadIdx.x & 31;
@@ -273,10 +276,11 @@ __global__ void __launch_bounds__(kCrThreads, kCrMinBlocks) hb_phase_kernel(cons
 }
 
 template <int MU, bool MEAS, bool SLAB = false, bool PEEL = true>
-static cudaError_t launch_hb(const HbParams &p, int device, cudaStream_t stream)
+static cudaError_t launch_hb(const HbParams &p, su2_lattice *lat)
 {
     static int blocks_per_sm[64] = {};
     static int num_sms[64] = {};
+    int device = lat->device;
     if (device < 0 || device >= 64) device = 0;
     if (!blocks_per_sm[device]) {
         cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm[device],
@@ -289,8 +293,9 @@ static cudaError_t launch_hb(const HbParams &p, int device, cudaStream_t stream)
     const int n = SLAB ? p.slab.eo_end - p.slab.eo_begin : p.g.vh;
     const int want = (n + kCrThreads - 1) / kCrThreads;
     const int grid = std::max(1, std::min(std::min(want, blocks_per_sm[device] * num_sms[device]), kFusedSlots));
-    if (PEEL && n > kCrPeelRounds * grid * kCrThreads) return launch_hb<MU, MEAS, SLAB, false>(p, device, stream);
-    hb_phase_kernel<MU, MEAS, SLAB, PEEL><<<grid, kCrThreads, 0, stream>>>(p);
+    if (PEEL && n > kCrPeelRounds * grid * kCrThreads) return launch_hb<MU, MEAS, SLAB, false>(p, lat);
+    if (MEAS) fused_launched(lat, MU, 0, grid);
+    hb_phase_kernel<MU, MEAS, SLAB, PEEL><<<grid, kCrThreads, 0, lat->stream>>>(p);
     return cudaGetLastError();
 }
 
@@ -314,16 +319,16 @@ su2_status launch_hb_phase(su2_lattice *lat, int mu, int parity, uint32_t sweep,
     cudaError_t e;
     if (p.plaq) {
         switch (mu) {
-        case 1: e = launch_hb<1, true>(p, lat->device, lat->stream); break;
-        case 2: e = launch_hb<2, true>(p, lat->device, lat->stream); break;
-        default: e = launch_hb<3, true>(p, lat->device, lat->stream); break;
+        case 1: e = launch_hb<1, true>(p, lat); break;
+        case 2: e = launch_hb<2, true>(p, lat); break;
+        default: e = launch_hb<3, true>(p, lat); break;
         }
     } else {
         switch (mu) {
-        case 0: e = launch_hb<0, false>(p, lat->device, lat->stream); break;
-        case 1: e = launch_hb<1, false>(p, lat->device, lat->stream); break;
-        case 2: e = launch_hb<2, false>(p, lat->device, lat->stream); break;
-        default: e = launch_hb<3, false>(p, lat->device, lat->stream); break;
+        case 0: e = launch_hb<0, false>(p, lat); break;
+        case 1: e = launch_hb<1, false>(p, lat); break;
+        case 2: e = launch_hb<2, false>(p, lat); break;
+        default: e = launch_hb<3, false>(p, lat); break;
         }
     }
     SU2_CUDA(e);
@@ -350,10 +355,10 @@ su2_status launch_hb_phase_slab(su2_lattice *lat, int mu, int parity_local, uint
     set_bases(p.same, p.other, lat, parity_local);
     cudaError_t e;
     switch (mu) {
-    case 0: e = launch_hb<0, false, true>(p, lat->device, lat->stream); break;
-    case 1: e = launch_hb<1, false, true>(p, lat->device, lat->stream); break;
-    case 2: e = launch_hb<2, false, true>(p, lat->device, lat->stream); break;
-    default: e = launch_hb<3, false, true>(p, lat->device, lat->stream); break;
+    case 0: e = launch_hb<0, false, true>(p, lat); break;
+    case 1: e = launch_hb<1, false, true>(p, lat); break;
+    case 2: e = launch_hb<2, false, true>(p, lat); break;
+    default: e = launch_hb<3, false, true>(p, lat); break;
     }
     SU2_CUDA(e);
     return SU2_OK;
@@ -553,8 +558,7 @@ static su2_status generation_graph(su2_lattice *lat, bool measure, bool reunit, 
     su2_status st = sweep_and_measure(lat, measure, reunit, lat->scratch.history,
                                       lat->scratch.history + lat->scratch.history_cap);
     if (st == SU2_OK) {
-        advance_kernel<<<1, 32, 0, lat->stream>>>(lat->d_ctr, measure ? 1 : 0);
-        if (cudaGetLastError() != cudaSuccess) st = SU2_E_CUDA;
+        if (!measure || reunit) st = enqueue_advance(lat, measure);  // otherwise the measurement's last kernel advances
     }
     lat->capturing = false;
     lat->sweep = sweep0;  // the captured sweep advanced the host counter; the replay does it

@@ -79,7 +79,10 @@ __global__ void __launch_bounds__(kKpThreads, kKpMinBlocks) kp_phase_kernel(cons
     const int eo_end = SLAB ? p.slab.eo_end : p.g.vh;
     const uint32_t rng_eo = SLAB ? p.slab.rng_eo : 0u;
     const uint32_t rng_parity = SLAB ? (uint32_t)p.slab.rng_parity : (uint32_t)p.parity;
-    if (p.gate != nullptr && *(volatile const unsigned int *)p.gate == 1u) return;
+    if (p.gate != nullptr && *(volatile const unsigned int *)p.gate == 1u) {
+        if (MEAS && threadIdx.x == 0) p.plaq[blockIdx.x] = 0.0;
+        return;
+    }
     __shared__ float4 s_ut[kKpWarps][kRetryCap];
     __shared__ float4 s_sp[MEAS ? kKpWarps : 1][kRetryCap];
     const uint32_t sweep = p.sweep_dev ? *p.sweep_dev : p.sweep;
@@ -265,10 +268,11 @@ __global__ void __launch_bounds__(kKpThreads, kKpMinBlocks) kp_phase_kernel(cons
 }
 
 template <int MU, bool MEAS, bool SLAB = false>
-static cudaError_t launch_kp(const KpParams &p, int device, cudaStream_t stream)
+static cudaError_t launch_kp(const KpParams &p, su2_lattice *lat)
 {
     static int per_sm[64] = {};
     static int sms[64] = {};
+    int device = lat->device;
     if (device < 0 || device >= 64) device = 0;
     if (!per_sm[device]) {
         cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[device],
@@ -280,7 +284,8 @@ static cudaError_t launch_kp(const KpParams &p, int device, cudaStream_t stream)
     const int n = SLAB ? p.slab.eo_end - p.slab.eo_begin : p.g.vh;
     const int want = (n + kKpThreads - 1) / kKpThreads;
     const int grid = std::max(1, std::min(std::min(want, per_sm[device] * sms[device]), kFusedSlots));
-    kp_phase_kernel<MU, MEAS, SLAB><<<grid, kKpThreads, 0, stream>>>(p);
+    if (MEAS) fused_launched(lat, MU, 0, grid);
+    kp_phase_kernel<MU, MEAS, SLAB><<<grid, kKpThreads, 0, lat->stream>>>(p);
     return cudaGetLastError();
 }
 
@@ -304,16 +309,16 @@ su2_status launch_kp_phase(su2_lattice *lat, int mu, int parity, uint32_t sweep,
     cudaError_t e;
     if (p.plaq) {
         switch (mu) {
-        case 1: e = launch_kp<1, true>(p, lat->device, lat->stream); break;
-        case 2: e = launch_kp<2, true>(p, lat->device, lat->stream); break;
-        default: e = launch_kp<3, true>(p, lat->device, lat->stream); break;
+        case 1: e = launch_kp<1, true>(p, lat); break;
+        case 2: e = launch_kp<2, true>(p, lat); break;
+        default: e = launch_kp<3, true>(p, lat); break;
         }
     } else {
         switch (mu) {
-        case 0: e = launch_kp<0, false>(p, lat->device, lat->stream); break;
-        case 1: e = launch_kp<1, false>(p, lat->device, lat->stream); break;
-        case 2: e = launch_kp<2, false>(p, lat->device, lat->stream); break;
-        default: e = launch_kp<3, false>(p, lat->device, lat->stream); break;
+        case 0: e = launch_kp<0, false>(p, lat); break;
+        case 1: e = launch_kp<1, false>(p, lat); break;
+        case 2: e = launch_kp<2, false>(p, lat); break;
+        default: e = launch_kp<3, false>(p, lat); break;
         }
     }
     SU2_CUDA(e);
@@ -340,10 +345,10 @@ su2_status launch_kp_phase_slab(su2_lattice *lat, int mu, int parity_local, uint
     set_bases(p.same, p.other, lat, parity_local);
     cudaError_t e;
     switch (mu) {
-    case 0: e = launch_kp<0, false, true>(p, lat->device, lat->stream); break;
-    case 1: e = launch_kp<1, false, true>(p, lat->device, lat->stream); break;
-    case 2: e = launch_kp<2, false, true>(p, lat->device, lat->stream); break;
-    default: e = launch_kp<3, false, true>(p, lat->device, lat->stream); break;
+    case 0: e = launch_kp<0, false, true>(p, lat); break;
+    case 1: e = launch_kp<1, false, true>(p, lat); break;
+    case 2: e = launch_kp<2, false, true>(p, lat); break;
+    default: e = launch_kp<3, false, true>(p, lat); break;
     }
     SU2_CUDA(e);
     return SU2_OK;

@@ -111,7 +111,10 @@ __global__ void __launch_bounds__(kLearnThreads, kLearnMinBlocks) learned_phase_
 {
     extern __shared__ __align__(16) float2 s_pairs[];
     __shared__ __align__(8) uint64_t s_bar;
-    if (*(volatile const unsigned int *)p.gate != 1u) return;
+    if (*(volatile const unsigned int *)p.gate != 1u) {
+        if (MEAS && threadIdx.x == 0) p.plaq[blockIdx.x] = 0.0;
+        return;
+    }
     // The table's row pairs come in by one bulk copy (the TMA engine) that
     // completes on an mbarrier, while the threads load their first staple.
     if (threadIdx.x == 0) {
@@ -164,7 +167,10 @@ __global__ void __launch_bounds__(kLearnThreads, kLearnMinBlocks) learned_phase_
         s_table_ok = ok ? 1 : 0;
     }
     __syncthreads();
-    if (!s_table_ok) return;  // block-uniform
+    if (!s_table_ok) {  // block-uniform
+        if (MEAS && threadIdx.x == 0) p.plaq[blockIdx.x] = 0.0;
+        return;
+    }
     tc::mbar_wait(&s_bar, 0, kTableWaitPolls);
     // a round; MORE: with the loads and the staple of the next one (the last
     // round of a warp runs without them)
@@ -277,7 +283,8 @@ __global__ void __launch_bounds__(kLearnThreads) collect_kernel(const float4 *__
 // Grid of all co-resident blocks (at most `want`), for the kernels that walk
 // their links in a loop.
 template <typename Kernel>
-static cudaError_t launch_persistent(Kernel kernel, const LearnedParams &p, int want, size_t smem, su2_lattice *lat)
+static cudaError_t launch_persistent(Kernel kernel, const LearnedParams &p, int mu, int want, size_t smem,
+                                     su2_lattice *lat)
 {
     int per_sm = 0, sms = 0;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -285,6 +292,7 @@ static cudaError_t launch_persistent(Kernel kernel, const LearnedParams &p, int 
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, lat->device);
     if (e != cudaSuccess) return e;
     const int grid = std::max(1, std::min(std::min(want, std::max(1, per_sm) * sms), kFusedSlots));
+    if (p.plaq) fused_launched(lat, mu, 1, grid);
     kernel<<<grid, kLearnThreads, smem, lat->stream>>>(p);
     return cudaGetLastError();
 }
@@ -322,16 +330,16 @@ static su2_status launch_learned_phase(su2_lattice *lat, int mu, int parity)
     cudaError_t e;
     if (p.plaq) {
         switch (mu) {
-        case 1: e = launch_persistent(learned_phase_kernel<1, true>, p, want, smem, lat); break;
-        case 2: e = launch_persistent(learned_phase_kernel<2, true>, p, want, smem, lat); break;
-        default: e = launch_persistent(learned_phase_kernel<3, true>, p, want, smem, lat); break;
+        case 1: e = launch_persistent(learned_phase_kernel<1, true>, p, mu, want, smem, lat); break;
+        case 2: e = launch_persistent(learned_phase_kernel<2, true>, p, mu, want, smem, lat); break;
+        default: e = launch_persistent(learned_phase_kernel<3, true>, p, mu, want, smem, lat); break;
         }
     } else {
         switch (mu) {
-        case 0: e = launch_persistent(learned_phase_kernel<0, false>, p, want, smem, lat); break;
-        case 1: e = launch_persistent(learned_phase_kernel<1, false>, p, want, smem, lat); break;
-        case 2: e = launch_persistent(learned_phase_kernel<2, false>, p, want, smem, lat); break;
-        default: e = launch_persistent(learned_phase_kernel<3, false>, p, want, smem, lat); break;
+        case 0: e = launch_persistent(learned_phase_kernel<0, false>, p, mu, want, smem, lat); break;
+        case 1: e = launch_persistent(learned_phase_kernel<1, false>, p, mu, want, smem, lat); break;
+        case 2: e = launch_persistent(learned_phase_kernel<2, false>, p, mu, want, smem, lat); break;
+        default: e = launch_persistent(learned_phase_kernel<3, false>, p, mu, want, smem, lat); break;
         }
     }
     SU2_CUDA(e);
@@ -418,7 +426,7 @@ static su2_status learned_graph(su2_lattice *lat, bool measure, double min_accep
     lat->capturing = true;
     su2_status st = learned_sweep_body(lat, measure, min_acceptance, lat->scratch.history,
                                        lat->scratch.history + lat->scratch.history_cap);
-    if (st == SU2_OK) st = enqueue_advance(lat, measure);
+    if (st == SU2_OK && !measure) st = enqueue_advance(lat, measure);  // a measured sweep's last kernel advances
     lat->capturing = false;
     cudaGraph_t graph = nullptr;
     const cudaError_t e = cudaStreamEndCapture(lat->stream, &graph);

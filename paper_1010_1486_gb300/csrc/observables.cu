@@ -94,19 +94,26 @@ constexpr int kPolySeg = 4;                  // warps per block: quarters of the
 constexpr int kPolyThreads = 32 * kPolySeg;  // block size
 constexpr int kPolyBatch = 12;               // loads in flight per lane (Nt = 48: one batch)
 
-// PLAQ: the kernel of a measuring sweep also sums the fused-plaquette slot
-// region `fused` (kFusedRegion doubles): block b adds its contiguous share in
-// index order, and the last block adds the block sums in block order into
-// plaq_dst (scaled by plaq_scale), beside the Polyakov loop; `partials` then
-// holds 2 gridDim.x doubles and must not overlap the slot region.
+// PLAQ: the kernel of a measuring sweep also sums the fused-plaquette slots
+// (fused.n[r] of region r): each block a share of every region, and the last
+// block the block sums in block order, into plaq_dst (scaled by plaq_scale),
+// beside the Polyakov loop; it then advances the counters of a graph replay
+// (ctr).  `partials` holds 2 gridDim.x doubles and must not
+// overlap the slots.
+struct FusedSlots {
+    const double *slots;
+    int n[6];
+};
+
 template <bool PLAQ>
 __global__ void __launch_bounds__(kPolyThreads) polyakov_kernel(const float4 *__restrict__ L, Geom g,
                                                                double *__restrict__ partials,
                                                                unsigned int *__restrict__ ticket,
                                                                double *__restrict__ dst,
                                                                const uint32_t *__restrict__ idx,
-                                                               const double *__restrict__ fused,
-                                                               double *__restrict__ plaq_dst, double plaq_scale)
+                                                               const FusedSlots fused,
+                                                               double *__restrict__ plaq_dst, double plaq_scale,
+                                                               uint32_t *__restrict__ ctr)
 {
     __shared__ float4 s_part[kPolySeg][32];
     float acc = 0.0f;  // per-thread partial in binary32; the block and grid sums are binary64
@@ -155,11 +162,11 @@ __global__ void __launch_bounds__(kPolyThreads) polyakov_kernel(const float4 *__
         finish_reduction(total_sum, partials, ticket, idx ? dst + *idx : dst, 1.0 / (double)g.vs);
         return;
     }
-    const int per = (kFusedRegion + (int)gridDim.x - 1) / (int)gridDim.x;
-    const int f0 = min((int)blockIdx.x * per, kFusedRegion);
-    const int f1 = min(f0 + per, kFusedRegion);
     double fv = 0.0;
-    for (int i = f0 + (int)threadIdx.x; i < f1; i += kPolyThreads) fv += fused[i];
+#pragma unroll
+    for (int r = 0; r < 6; ++r)
+        for (int i = (int)blockIdx.x * kPolyThreads + (int)threadIdx.x; i < fused.n[r]; i += (int)gridDim.x * kPolyThreads)
+            fv += fused.slots[r * kFusedSlots + i];
     const double fused_sum = block_sum(fv);
     __shared__ bool last;
     if (threadIdx.x == 0) {
@@ -179,10 +186,14 @@ __global__ void __launch_bounds__(kPolyThreads) polyakov_kernel(const float4 *__
     vp = block_sum(vp);
     vq = block_sum(vq);
     if (threadIdx.x == 0) {
-        const uint32_t slot = idx ? *idx : 0u;
+        const uint32_t slot = ctr ? ctr[1] : 0u;
         dst[slot] = vp * (1.0 / (double)g.vs);
         plaq_dst[slot] = vq * plaq_scale;
         *ticket = 0u;
+        if (ctr) {
+            ctr[0] += 1u;
+            ctr[1] = slot + 1u;
+        }
     }
 }
 
@@ -209,8 +220,8 @@ su2_status fused_begin(su2_lattice *lat)
         set_last_error("reduction scratch too small for the fused plaquette");
         return SU2_E_INVAL;
     }
-    SU2_CUDA(cudaMemsetAsync(lat->scratch.partials, 0, sizeof(double) * kFusedRegion, lat->stream));
     lat->fused_part = lat->scratch.partials;
+    for (int &n : lat->fused_blocks) n = 0;
     return SU2_OK;
 }
 
@@ -221,7 +232,7 @@ su2_status launch_polyakov(su2_lattice *lat, double *dst)
     polyakov_kernel<false><<<grid, kPolyThreads, 0, lat->stream>>>(lat->links, g, lat->scratch.partials,
                                                                      lat->scratch.ticket + 1, dst,
                                                                      lat->capturing ? lat->d_ctr + 1 : nullptr,
-                                                                     nullptr, nullptr, 0.0);
+                                                                     FusedSlots(), nullptr, 0.0, nullptr);
     SU2_CUDA(cudaGetLastError());
     return SU2_OK;
 }
@@ -235,9 +246,12 @@ su2_status fused_finish_with_polyakov(su2_lattice *lat, double *plaq_dst, double
         return SU2_E_INVAL;
     }
     lat->fused_part = nullptr;
+    FusedSlots fused;
+    fused.slots = lat->scratch.partials;
+    std::copy(lat->fused_blocks, lat->fused_blocks + 6, fused.n);
     polyakov_kernel<true><<<grid, kPolyThreads, 0, lat->stream>>>(
-        lat->links, g, lat->scratch.partials + kFusedRegion, lat->scratch.ticket + 1, poly_dst,
-        lat->capturing ? lat->d_ctr + 1 : nullptr, lat->scratch.partials, plaq_dst, 1.0 / (6.0 * (double)lat->vol));
+        lat->links, g, lat->scratch.partials + kFusedRegion, lat->scratch.ticket + 1, poly_dst, nullptr, fused, plaq_dst,
+        1.0 / (6.0 * (double)lat->vol), lat->capturing ? lat->d_ctr : nullptr);
     SU2_CUDA(cudaGetLastError());
     return SU2_OK;
 }

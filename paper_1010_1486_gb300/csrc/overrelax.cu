@@ -115,10 +115,11 @@ __global__ void __launch_bounds__(kOrThreads, kOrMinBlocks) or_phase_kernel(cons
 }
 
 template <int MU, bool MEAS, bool PEEL = true>
-static cudaError_t launch_or(const OrParams &p, int device, cudaStream_t stream)
+static cudaError_t launch_or(const OrParams &p, su2_lattice *lat)
 {
     static int per_sm[64] = {};
     static int sms[64] = {};
+    int device = lat->device;
     if (device < 0 || device >= 64) device = 0;
     if (!per_sm[device]) {
         cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[device],
@@ -129,8 +130,9 @@ static cudaError_t launch_or(const OrParams &p, int device, cudaStream_t stream)
     }
     const int want = (p.g.vh + kOrThreads - 1) / kOrThreads;
     const int grid = std::max(1, std::min(std::min(want, per_sm[device] * sms[device]), kFusedSlots));
-    if (PEEL && p.g.vh > kOrPeelRounds * grid * kOrThreads) return launch_or<MU, MEAS, false>(p, device, stream);
-    or_phase_kernel<MU, MEAS, PEEL><<<grid, kOrThreads, 0, stream>>>(p);
+    if (PEEL && p.g.vh > kOrPeelRounds * grid * kOrThreads) return launch_or<MU, MEAS, false>(p, lat);
+    if (MEAS) fused_launched(lat, MU, 0, grid);
+    or_phase_kernel<MU, MEAS, PEEL><<<grid, kOrThreads, 0, lat->stream>>>(p);
     return cudaGetLastError();
 }
 
@@ -145,16 +147,16 @@ su2_status launch_or_phase(su2_lattice *lat, int mu, int parity)
     cudaError_t e;
     if (p.plaq) {
         switch (mu) {
-        case 1: e = launch_or<1, true>(p, lat->device, lat->stream); break;
-        case 2: e = launch_or<2, true>(p, lat->device, lat->stream); break;
-        default: e = launch_or<3, true>(p, lat->device, lat->stream); break;
+        case 1: e = launch_or<1, true>(p, lat); break;
+        case 2: e = launch_or<2, true>(p, lat); break;
+        default: e = launch_or<3, true>(p, lat); break;
         }
     } else {
         switch (mu) {
-        case 0: e = launch_or<0, false>(p, lat->device, lat->stream); break;
-        case 1: e = launch_or<1, false>(p, lat->device, lat->stream); break;
-        case 2: e = launch_or<2, false>(p, lat->device, lat->stream); break;
-        default: e = launch_or<3, false>(p, lat->device, lat->stream); break;
+        case 0: e = launch_or<0, false>(p, lat); break;
+        case 1: e = launch_or<1, false>(p, lat); break;
+        case 2: e = launch_or<2, false>(p, lat); break;
+        default: e = launch_or<3, false>(p, lat); break;
         }
     }
     SU2_CUDA(e);

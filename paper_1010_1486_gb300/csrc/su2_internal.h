@@ -19,7 +19,8 @@ constexpr int kHbThreads = 128;      // block size of the heat-bath phase kernel
 // Plaquette measured during a sweep: the odd phases of mu = 1, 2, 3 each add
 // the plaquettes of planes (nu, mu), nu < mu, through the new links; block
 // partials go to slots [(mu - 1) * 2 + kind] * kFusedSlots + block (kind 0:
-// heat bath / over-relaxation, 1: learned), zero-filled first.
+// heat bath / over-relaxation, 1: learned; a kernel that its gate turns away
+// writes zeros), and the sum takes the slots of the blocks that were launched.
 constexpr int kFusedSlots = 1024;
 constexpr int kFusedRegion = 6 * kFusedSlots;
 
@@ -74,6 +75,7 @@ struct su2_lattice {
 
     int overrelax = 0;  // over-relaxation sweeps after each heat-bath sweep
     double *fused_part = nullptr;  // slot region of the plaquette measured in the current sweep, or NULL
+    int fused_blocks[6] = {};      // blocks of the measuring launches, by [(mu - 1) * 2 + kind]
     bool capturing = false;        // launches are being captured into a generation graph
     bool graphs_off = false;       // a capture failed once: generate eagerly
     uint32_t *d_ctr = nullptr;     // device: [0] sweep counter, [1] measurement slot (graph replays)
@@ -234,11 +236,16 @@ inline double *fused_slot(const su2_lattice *lat, int mu, int parity, int kind)
     if (!lat->fused_part || parity != 1 || mu < 1) return nullptr;
     return lat->fused_part + ((mu - 1) * 2 + kind) * kFusedSlots;
 }
-// Zero-fills the slot region and points the lattice at it (the next sweep
-// measures); fused_finish_with_polyakov detaches it and, in one launch, sums
-// the region (block shares in index order, then the shares in block order)
-// into *plaq_dst (device) scaled to the mean plaquette, and writes the
-// Polyakov loop to *poly_dst.
+// What a launcher calls with its grid when it measures.
+inline void fused_launched(su2_lattice *lat, int mu, int kind, int blocks)
+{
+    lat->fused_blocks[(mu - 1) * 2 + kind] = blocks;
+}
+// Points the lattice at the slot region (the next sweep measures);
+// fused_finish_with_polyakov detaches it and, in one launch, sums the launched
+// blocks' slots (block shares, then the shares in block order) into *plaq_dst
+// (device) scaled to the mean plaquette, writes the Polyakov loop to *poly_dst
+// and, in a captured sweep, advances the device counters.
 su2_status fused_begin(su2_lattice *lat);
 // Graph replays of generation loops: the device sweep counter and measurement
 // slot set from the host state (one-thread kernel), advanced at the end of a
