@@ -171,38 +171,31 @@ __device__ void batch_phase(const BatchParams &bp, int parity, uint32_t sweep, C
         int retry_n = 0, done_n = 0;
         float plaq = 0.0f;  // per-thread partial in binary32; the block and grid sums are binary64
 
-        // lanes that push nothing write to the last slot, which no live entry
-        // reaches (at most 31 left over + 32 pushed), so the stores need no branch
-        auto push_done = [&](bool ok, float4 ut, float val, float ibk, int eo, float4 sp) {
-            const unsigned int m = __ballot_sync(0xffffffffu, ok);
-            const int q = ok ? done_n + __popc(m & lanes_below) : kCrQueue - 1;
-            Q.d_ut[q] = ut;
-            Q.d_val[q] = val;
-            Q.d_ibk[q] = ibk;
-            Q.d_eo[q] = eo;
-            if (MEAS) Q.d_sp[q] = sp;
-            done_n += __popc(m);
-        };
-        auto push_retry = [&](bool again, float4 ut, float ibk, float e, int eo, int blk, float4 sp) {
-            const unsigned int m = __ballot_sync(0xffffffffu, again);
-            const int q = again ? retry_n + __popc(m & lanes_below) : kCrQueue - 1;
-            Q.r_ut[q] = ut;
-            Q.r_ibk[q] = ibk;
-            Q.r_e[q] = e;
-            Q.r_eo[q] = eo;
-            Q.r_blk[q] = blk;
-            if (MEAS) Q.r_sp[q] = sp;
-            retry_n += __popc(m);
+        // lanes with `in` join the direction queue (ok; x = val) or the retry
+        // queue (x = e)
+        auto push = [&](bool in, bool ok, float4 ut, float ibk, float x, int eo, int blk, float4 sp) {
+            const unsigned int m_ok = __ballot_sync(0xffffffffu, in && ok);
+            const unsigned int m_again = __ballot_sync(0xffffffffu, in && !ok);
+            const int rank = __popc((ok ? m_ok : m_again) & lanes_below);
+            const int q = !in ? kCrNobody : ok ? done_n + rank : kCrRetryTop - retry_n - rank;
+            Q.ut[q] = ut;
+            Q.ibk[q] = ibk;
+            Q.x[q] = x;
+            Q.eo[q] = eo;
+            Q.blk[q] = blk;
+            if (MEAS) Q.sp[q] = sp;
+            done_n += __popc(m_ok);
+            retry_n += __popc(m_again);
         };
         auto direction_pass = [&](int first, int n) {
             __syncwarp();
             if (lane < n) {
                 const int q = first + lane;
-                const int eo = Q.d_eo[q];
+                const int eo = Q.eo[q];
                 const uint4 wd = philox_key(make_uint4(direction_pair((uint32_t)eo), sweep, sw_dir, 0u), k0, k1);
-                const float4 out = direction_update(deferred_a0(Q.d_val[q], Q.d_ibk[q]), Q.d_ut[q], wd, (uint32_t)eo);
+                const float4 out = direction_update(deferred_a0(Q.x[q], Q.ibk[q]), Q.ut[q], wd, (uint32_t)eo);
                 links[link_index(g, MU, parity, eo)] = out;
-                if (MEAS) plaq = __fadd_rn(plaq, qmul_re(out, Q.d_sp[q]));
+                if (MEAS) plaq = __fadd_rn(plaq, qmul_re(out, Q.sp[q]));
             }
             __syncwarp();
         };
@@ -219,13 +212,13 @@ __device__ void batch_phase(const BatchParams &bp, int parity, uint32_t sweep, C
             float ibk = 1.0f, e = 0.0f;
             int eo = 0, blk = 0;
             if (have) {
-                const int q = first + lane;
-                ut = Q.r_ut[q];
-                ibk = Q.r_ibk[q];
-                e = Q.r_e[q];
-                eo = Q.r_eo[q];
-                blk = Q.r_blk[q];
-                if (MEAS) sp = Q.r_sp[q];
+                const int q = kCrRetryTop - (first + lane);
+                ut = Q.ut[q];
+                ibk = Q.ibk[q];
+                e = Q.x[q];
+                eo = Q.eo[q];
+                blk = Q.blk[q];
+                if (MEAS) sp = Q.sp[q];
             }
             __syncwarp();
             const uint4 w = philox_key(make_uint4((uint32_t)eo, sweep, sw_creutz, (uint32_t)blk), k0, k1);
@@ -243,8 +236,7 @@ __device__ void batch_phase(const BatchParams &bp, int parity, uint32_t sweep, C
                     my_trials += (unsigned int)kMaxTrials;
                 }
             }
-            push_retry(again, ut, ibk, e, eo, blk + 1, sp);
-            push_done(ok, ut, val, ibk, eo, sp);
+            push(ok || again, ok, ut, ibk, ok ? val : e, eo, blk + 1, sp);
             flush_done();
         };
 
@@ -286,8 +278,7 @@ __device__ void batch_phase(const BatchParams &bp, int parity, uint32_t sweep, C
                 const bool acc = creutz_pair(w, ds.ibk, ds.e, valid, first_ok, val);
                 const bool ok = valid && acc;
                 my_trials += ok ? (first_ok ? 1u : 2u) : 0u;
-                push_done(ok, ds.ut, val, ds.ibk, cur, sp_cur);
-                push_retry(valid && !acc, ds.ut, ds.ibk, ds.e, cur, 1, sp_cur);
+                push(valid, ok, ds.ut, ds.ibk, ok ? val : ds.e, cur, 1, sp_cur);
             }
             if (more) v_next = add_nu_terms(v_next, nl);
             if (MU == 2) sp_next = v_next;

@@ -65,9 +65,9 @@ __device__ void batch_phase_kp(const BatchParams &bp, int parity, uint32_t sweep
         auto retry = [&](int first, int n) {
             if (lane < n) {
                 const int q = first + lane;
-                float4 ut = Q.r_ut[q];
-                float bk_q = Q.r_ibk[q];
-                const int eo = Q.r_eo[q];
+                float4 ut = Q.ut[q];
+                float bk_q = Q.ibk[q];
+                const int eo = Q.eo[q];
                 float a0 = 0.0f;
                 int t = 1;
                 if (!(bk_q >= min_bk && bk_q <= kKpMaxBk)) {
@@ -86,7 +86,7 @@ __device__ void batch_phase_kp(const BatchParams &bp, int parity, uint32_t sweep
                     const int nt = heatbath_draw_gen(ut, beta, gen, (uint32_t)eo, sweep, (uint32_t)parity, MU, out);
                     if (nt > 0) {
                         links[link_index(g, MU, parity, eo)] = out;
-                        if (MEAS) plaq = __fadd_rn(plaq, qmul_re(out, Q.r_sp[q]));
+                        if (MEAS) plaq = __fadd_rn(plaq, qmul_re(out, Q.sp[q]));
                         my_trials += (unsigned int)nt;
                     } else {
                         atomicAdd(&bp.flags[0], 1u);
@@ -103,7 +103,7 @@ __device__ void batch_phase_kp(const BatchParams &bp, int parity, uint32_t sweep
                     const float4 out = direction_update(
                         a0, ut, gen(make_uint4(direction_pair((uint32_t)eo), sweep, sw_dir, 0u)), (uint32_t)eo);
                     links[link_index(g, MU, parity, eo)] = out;
-                    if (MEAS) plaq = __fadd_rn(plaq, qmul_re(out, Q.r_sp[q]));
+                    if (MEAS) plaq = __fadd_rn(plaq, qmul_re(out, Q.sp[q]));
                     my_trials += (unsigned int)(t + 1);
                 } else {
                     atomicAdd(&bp.flags[0], 1u);  // trial cap: the link keeps its old value
@@ -168,10 +168,10 @@ __device__ void batch_phase_kp(const BatchParams &bp, int parity, uint32_t sweep
             const unsigned int parked = __ballot_sync(0xffffffffu, park);
             if (park) {  // rare at large beta k: a branch costs less than stores from every lane
                 const int q = queued + __popc(parked & lanes_below);
-                Q.r_ut[q] = use_kp ? ut : v_cur;
-                Q.r_ibk[q] = bk;
-                Q.r_eo[q] = cur;
-                if (MEAS) Q.r_sp[q] = sp_cur;
+                Q.ut[q] = use_kp ? ut : v_cur;
+                Q.ibk[q] = bk;
+                Q.eo[q] = cur;
+                if (MEAS) Q.sp[q] = sp_cur;
             }
             queued += __popc(parked);
             if (more) v_next = add_nu_terms(v_next, nl);

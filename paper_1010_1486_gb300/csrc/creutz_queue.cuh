@@ -8,22 +8,21 @@
 
 namespace su2 {
 
-constexpr int kCrQueue = 64;  // per warp and queue: at most 31 left over + 32 pushed at once
+// Both queues share one array: the direction queue grows from its start, the
+// retry queue from kCrRetryTop down.  A push finds at most 31 entries in each
+// and adds at most 32 in all, so 94 hold them; lanes that push nothing write to
+// entry kCrNobody, which nobody reads, so the stores need no branch.
+constexpr int kCrRetryTop = 93;
+constexpr int kCrNobody = 94;
+constexpr int kCrEntries = 95;
 
 struct CrQueues {
-    // links still without an accepted trial: U~^dag, 1/(beta k) (0 on the Haar
-    // branch), exp(-2 beta k), index, next Philox block
-    float4 r_ut[kCrQueue];
-    float r_ibk[kCrQueue], r_e[kCrQueue];
-    int r_eo[kCrQueue], r_blk[kCrQueue];
-    // links with an accepted trial waiting for their a0, direction and store:
-    // U~^dag, x of the trial (a0 on the Haar branch), 1/(beta k), index
-    float4 d_ut[kCrQueue];
-    float d_val[kCrQueue], d_ibk[kCrQueue];
-    int d_eo[kCrQueue];
-    // when the phase measures the plaquette: the link's staple terms of the
-    // directions nu < mu, for the retry and the direction queue
-    float4 r_sp[kCrQueue], d_sp[kCrQueue];
+    float4 ut[kCrEntries];  // U~^dag
+    float ibk[kCrEntries];  // 1/(beta k) (0 on the Haar branch); beta k for Kennedy-Pendleton
+    float x[kCrEntries];    // waiting for a trial: exp(-2 beta k); accepted: x of the trial (a0 on the Haar branch)
+    int eo[kCrEntries], blk[kCrEntries];  // index, next Philox block
+    // when the phase measures the plaquette: the staple terms of the directions nu < mu
+    float4 sp[kCrEntries];
 };
 
 }  // namespace su2

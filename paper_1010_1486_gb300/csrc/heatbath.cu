@@ -57,7 +57,8 @@ constexpr int kCrMinBlocks = SU2_HB_MIN_BLOCKS;  // blocks per SM the register b
 //   part 0  k, U~^dag, beta k, exp(-2 beta k); Philox block 0 (trials 0, 1);
 //   part 1  trials 0 and 1, screened (creutz_pair); an accepted link goes to
 //           the warp's direction queue, a link with both rejected to its
-//           retry queue;
+//           retry queue (one array, one store per link: 3% at 48^4 against a
+//           store to either queue);
 //   part 2  every 32 links in the direction queue: a0 (the one exact log of
 //           the link), directions and stores.
 // Whenever 32 links wait for a retry, the whole warp draws their next Philox
@@ -111,41 +112,33 @@ __global__ void __launch_bounds__(kCrThreads, kCrMinBlocks) hb_phase_kernel(cons
     float plaq = 0.0f;  // per-thread partial in binary32; the block and grid sums are binary64
     int retry_n = 0, done_n = 0;  // warp-uniform queue lengths
 
-    // Lanes that push nothing write to the last slot, which no live entry
-    // reaches (at most 31 left over + 32 pushed = 63), so the stores need no
-    // branch.
-    auto push_done = [&](bool ok, float4 ut, float val, float ibk, int eo, float4 sp) {
-        const unsigned int m = __ballot_sync(0xffffffffu, ok);
-        const int q = ok ? done_n + __popc(m & lanes_below) : kCrQueue - 1;
-        Q.d_ut[q] = ut;
-        Q.d_val[q] = val;
-        Q.d_ibk[q] = ibk;
-        Q.d_eo[q] = eo;
-        if (MEAS) Q.d_sp[q] = sp;
-        done_n += __popc(m);
-    };
-    auto push_retry = [&](bool again, float4 ut, float ibk, float e, int eo, int blk, float4 sp) {
-        const unsigned int m = __ballot_sync(0xffffffffu, again);
-        const int q = again ? retry_n + __popc(m & lanes_below) : kCrQueue - 1;
-        Q.r_ut[q] = ut;
-        Q.r_ibk[q] = ibk;
-        Q.r_e[q] = e;
-        Q.r_eo[q] = eo;
-        Q.r_blk[q] = blk;
-        if (MEAS) Q.r_sp[q] = sp;
-        retry_n += __popc(m);
+    // lanes with `in` join the direction queue (ok; x = val) or the retry
+    // queue (x = e)
+    auto push = [&](bool in, bool ok, float4 ut, float ibk, float x, int eo, int blk, float4 sp) {
+        const unsigned int m_ok = __ballot_sync(0xffffffffu, in && ok);
+        const unsigned int m_again = __ballot_sync(0xffffffffu, in && !ok);
+        const int rank = __popc((ok ? m_ok : m_again) & lanes_below);
+        const int q = !in ? kCrNobody : ok ? done_n + rank : kCrRetryTop - retry_n - rank;
+        Q.ut[q] = ut;
+        Q.ibk[q] = ibk;
+        Q.x[q] = x;
+        Q.eo[q] = eo;
+        Q.blk[q] = blk;
+        if (MEAS) Q.sp[q] = sp;
+        done_n += __popc(m_ok);
+        retry_n += __popc(m_again);
     };
     // directions and stores of direction-queue entries [first, first + n)
     auto direction_pass = [&](int first, int n) {
         __syncwarp();
         if (lane < n) {
             const int q = first + lane;
-            const int eo = Q.d_eo[q];
+            const int eo = Q.eo[q];
             const uint32_t eo_g = (uint32_t)eo + rng_eo;
             const uint4 wd = philox_rk(make_uint4(direction_pair(eo_g), sweep, sw_dir, 0u), p.rk);
-            const float4 out = direction_update(deferred_a0(Q.d_val[q], Q.d_ibk[q]), Q.d_ut[q], wd, eo_g);
+            const float4 out = direction_update(deferred_a0(Q.x[q], Q.ibk[q]), Q.ut[q], wd, eo_g);
             p.links[link_index(p.g, MU, p.parity, eo)] = out;
-            if (MEAS) plaq = __fadd_rn(plaq, qmul_re(out, Q.d_sp[q]));
+            if (MEAS) plaq = __fadd_rn(plaq, qmul_re(out, Q.sp[q]));
         }
         __syncwarp();
     };
@@ -163,13 +156,13 @@ __global__ void __launch_bounds__(kCrThreads, kCrMinBlocks) hb_phase_kernel(cons
         float ibk = 1.0f, e = 0.0f;
         int eo = 0, blk = 0;
         if (have) {
-            const int q = first + lane;
-            ut = Q.r_ut[q];
-            ibk = Q.r_ibk[q];
-            e = Q.r_e[q];
-            eo = Q.r_eo[q];
-            blk = Q.r_blk[q];
-            if (MEAS) sp = Q.r_sp[q];
+            const int q = kCrRetryTop - (first + lane);
+            ut = Q.ut[q];
+            ibk = Q.ibk[q];
+            e = Q.x[q];
+            eo = Q.eo[q];
+            blk = Q.blk[q];
+            if (MEAS) sp = Q.sp[q];
         }
         __syncwarp();
         const uint4 w = philox_rk(make_uint4((uint32_t)eo + rng_eo, sweep, sw_creutz, (uint32_t)blk), p.rk);
@@ -188,8 +181,7 @@ __global__ void __launch_bounds__(kCrThreads, kCrMinBlocks) hb_phase_kernel(cons
                 trials += (unsigned int)(2 * p.max_blocks);
             }
         }
-        push_retry(again, ut, ibk, e, eo, blk + 1, sp);
-        push_done(ok, ut, val, ibk, eo, sp);
+        push(ok || again, ok, ut, ibk, ok ? val : e, eo, blk + 1, sp);
         flush_done();
     };
 
@@ -231,8 +223,7 @@ __global__ void __launch_bounds__(kCrThreads, kCrMinBlocks) hb_phase_kernel(cons
             const bool acc = creutz_pair(w, d.ibk, d.e, valid, first_ok, val);
             const bool ok = valid && acc;
             trials += ok ? (first_ok ? 1u : 2u) : 0u;
-            push_done(ok, d.ut, val, d.ibk, cur, sp_cur);
-            push_retry(valid && !acc, d.ut, d.ibk, d.e, cur, 1, sp_cur);
+            push(valid, ok, d.ut, d.ibk, ok ? val : d.e, cur, 1, sp_cur);
         }
         if constexpr (MORE) v_next = add_nu_terms(v_next, nl);
         if (MU == 2) sp_next = v_next;

@@ -29,7 +29,7 @@ __global__ void math_selftest_kernel(int which, const float *__restrict__ x, flo
         } else if (which == 1) {
             y[i] = exp_series(x[i]);
         } else if (which == 3) {
-            y[i] = __log2f(x[i]);
+            y[i] = log2_approx(x[i]);
         } else if (which == 4) {
             // quadruple (r1, r2, 1/(beta k), exp(-2 beta k)): the screen's
             // verdict and the exact test's
