@@ -27,6 +27,34 @@ __device__ __forceinline__ double block_sum(double v)
     return v;
 }
 
+// block_sum of two values side by side (each with block_sum's order of
+// additions): one chain of binary64 additions and one barrier instead of two.
+// Not called twice without a barrier in between.
+__device__ __forceinline__ void block_sum2(double &a, double &b)
+{
+    __shared__ double2 warp_sums[32];
+    const unsigned int lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, off);
+        b += __shfl_down_sync(0xffffffffu, b, off);
+    }
+    if (lane == 0) warp_sums[warp] = make_double2(a, b);
+    __syncthreads();
+    a = b = 0.0;
+    if (warp == 0) {
+        if (lane < blockDim.x >> 5) {
+            a = warp_sums[lane].x;
+            b = warp_sums[lane].y;
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            a += __shfl_down_sync(0xffffffffu, a, off);
+            b += __shfl_down_sync(0xffffffffu, b, off);
+        }
+    }
+}
+
 // Sum over the six planes mu < nu, in the order (0,1),(0,2),(0,3),(1,2),(1,3),
 // (2,3), of (1/2) Tr U_mu(x) U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag.
 template <bool NC = true>
