@@ -245,7 +245,7 @@ __device__ __forceinline__ bool metropolis_exact(float bk, float a_new, float ac
     return delta >= 0.0f || u1 <= exp_neg(delta);
 }
 
-// The same verdict screened with the hardware base-2 logarithm (__log2f:
+// The same verdict screened with the hardware base-2 logarithm (log2_approx:
 // absolute error <= 2^-22 on [1/2, 2], relative <= 2.4e-7 elsewhere; checked
 // with the Creutz screen).  With N, D the ratio's numerator and denominator
 // and l = (1/2) ln(N/D), the exact log(ratio) is within 2e-7 + 1e-6 |l| of l
@@ -266,13 +266,13 @@ __device__ __forceinline__ int metropolis_screen(float bk, float a_new, float ac
     const float num = __fmul_rn(one_new, __fmul_rn(fp_new, fp_new));
     const float den = __fmul_rn(one_cur, __fmul_rn(fp_cur, fp_cur));
     if (!(num > 1e-30f && num < 1e30f && den > 1e-30f && den < 1e30f)) return kScreenUndecided;
-    const float lg_n = __log2f(num), lg_d = __log2f(den);
+    const float lg_n = log2_approx(num), lg_d = log2_approx(den);
     const float lr = __fmul_rn(0.346573591f, __fsub_rn(lg_n, lg_d));
     const float dt = __fmaf_rn(bk, __fsub_rn(a_new, acur), lr);
     const float slack = __fmaf_rn(4e-6f, __fadd_rn(fabsf(lg_n), fabsf(lg_d)), 2e-4f);
     if (dt > slack) return kScreenAccept;
     if (!(dt < -slack)) return kScreenUndecided;
-    const float lu = __fmul_rn(0.693147182f, __log2f(u1));
+    const float lu = __fmul_rn(0.693147182f, log2_approx(u1));
     const float slack2 = __fmaf_rn(1e-6f, -dt, __fadd_rn(slack, 1e-5f));
     if (lu < __fsub_rn(dt, slack2)) return kScreenAccept;
     if (lu > __fadd_rn(dt, slack2)) return kScreenReject;
