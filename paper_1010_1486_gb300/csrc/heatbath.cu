@@ -83,7 +83,8 @@ constexpr int kCrMinBlocks = SU2_HB_MIN_BLOCKS;  // blocks per SM the register b
 // is the slower one.  us per phase with and without, measured every sweep,
 // beta = 4: 20^4 14.3 / 15.7, 24^4 17.9 / 19.4, 32^4 30.8 / 32.0, 36^4 (7.2
 // rounds) 44.8 / 45.5, 40^4 (11) 61.3 / 61.5, 44^4 83.8 / 83.2, 48^4 (22.7)
-// 113.6 / 111.8; so up to kCrPeelRounds.
+// 113.6 / 111.8 (all with separate queues; one array has since taken 1 us off
+// both at 24^4 and 3 at 48^4); so up to kCrPeelRounds.
 constexpr int kCrPeelRounds = 10;
 
 template <int MU, bool MEAS, bool SLAB, bool PEEL>

@@ -43,7 +43,9 @@ constexpr int kWilsonMaxT = 64;
 // *flag, and the host then takes the binary64 path.
 // Bound: instruction issue (71% of the slots; 82 warp instructions per 32
 // loops, the tile's preparation included).  24^4, all loops up to 8 x 8: 1243
-// -> 219 us per call, of it 189 us (ncu) in this kernel.
+// -> 217 us per call, of it 189 us (ncu) in this kernel.  Fewer instructions
+// alone do not help: loops in pairs (R, R + 1) with packed multiply-adds took
+// 205 to 246 us at 24^4 and 3% more at 48^4.
 constexpr int kLoopChunk = 8;          // extents R and T per block
 constexpr int kTileThreads = 256;      // most sites of a tile
 constexpr int kTileMaxBx = 64;         // most columns of a tile
