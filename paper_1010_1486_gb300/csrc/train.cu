@@ -198,7 +198,11 @@ struct Smem {
 
 // Dependent launches (the step and the Adam kernel alternate): let the next
 // grid of the stream start its independent prologue, and wait until the
-// previous grid has finished and its writes are visible.
+// previous grid has finished and its writes are visible.  A grid is resident
+// while earlier ones still write what it will read after the wait, so these
+// reads (operand tiles, weights, Adam state, partial sums) are not of data that
+// is constant for the grid's lifetime: they take __ldcg, which reads L2, and
+// never the non-coherent path that a const __restrict__ pointer would allow.
 __device__ __forceinline__ void release_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -437,12 +441,12 @@ __global__ void __launch_bounds__(kTrainThreads) train_step_kernel(const StepPar
     const float2 pr = p.pairs[idx];
     wait_previous_grid();
 
-    ((uint4 *)sm.W2)[t] = p.images[t];
-    if (warp == 0) sm.w1[lane] = w[learned::kOffW1 + lane];
-    if (warp == 1) sm.b1[lane] = w[learned::kOffB1 + lane];
-    if (warp == 2) sm.b2[lane] = w[learned::kOffB2 + lane];
-    if (warp == 3) sm.b3[lane] = lane < learned::kOut ? w[learned::kOffB3 + lane] : 0.0f;
-    const float s = (pr.x - w[learned::kOffMean]) * w[learned::kOffScale];
+    ((uint4 *)sm.W2)[t] = __ldcg(p.images + t);
+    if (warp == 0) sm.w1[lane] = __ldcg(w + learned::kOffW1 + lane);
+    if (warp == 1) sm.b1[lane] = __ldcg(w + learned::kOffB1 + lane);
+    if (warp == 2) sm.b2[lane] = __ldcg(w + learned::kOffB2 + lane);
+    if (warp == 3) sm.b3[lane] = lane < learned::kOut ? __ldcg(w + learned::kOffB3 + lane) : 0.0f;
+    const float s = (pr.x - __ldcg(w + learned::kOffMean)) * __ldcg(w + learned::kOffScale);
     const float a = fminf(fmaxf(pr.y, -1.0f), 1.0f);
     if (part == 0) sm.s_in[row] = s;
     tc::fence_before_sync();
@@ -532,10 +536,9 @@ __global__ void __launch_bounds__(kTrainThreads) train_step_kernel(const StepPar
 
 // Sums the per-CTA partials (in CTA order) into the mean gradient and loss;
 // with lr > 0 also applies one Adam step to the master weights.
-__global__ void adam_kernel(float *__restrict__ w, float *__restrict__ m, float *__restrict__ v,
-                            const float *__restrict__ partials, int nblocks, float inv_batch, float lr, float b1,
-                            float b2, float eps, float bias1, float bias2, float *__restrict__ grad_out,
-                            float *__restrict__ loss_out, unsigned char *__restrict__ images)
+__global__ void adam_kernel(float *w, float *m, float *v, const float *partials, int nblocks, float inv_batch,
+                            float lr, float b1, float b2, float eps, float bias1, float bias2, float *grad_out,
+                            float *loss_out, unsigned char *images)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     release_next_grid();
@@ -543,7 +546,7 @@ __global__ void adam_kernel(float *__restrict__ w, float *__restrict__ m, float 
     if (i >= kGradSlots) return;
     float gsum = 0.0f;
 #pragma unroll 16
-    for (int b = 0; b < nblocks; ++b) gsum += partials[(size_t)b * kGradSlots + i];
+    for (int b = 0; b < nblocks; ++b) gsum += __ldcg(partials + (size_t)b * kGradSlots + i);
     const float g = gsum * inv_batch;
     if (i == learned::kTrainable) {
         if (loss_out) *loss_out = g;
@@ -551,11 +554,11 @@ __global__ void adam_kernel(float *__restrict__ w, float *__restrict__ m, float 
     }
     if (grad_out) grad_out[i] = g;
     if (lr > 0.0f) {
-        const float mi = b1 * m[i] + (1.0f - b1) * g;
-        const float vi = b2 * v[i] + (1.0f - b2) * g * g;
+        const float mi = b1 * __ldcg(m + i) + (1.0f - b1) * g;
+        const float vi = b2 * __ldcg(v + i) + (1.0f - b2) * g * g;
         m[i] = mi;
         v[i] = vi;
-        const float wi = w[i] - lr * (mi / bias1) / (sqrtf(vi / bias2) + eps);
+        const float wi = __ldcg(w + i) - lr * (mi / bias1) / (sqrtf(vi / bias2) + eps);
         w[i] = wi;
         put_images(images, i, wi);
     }

@@ -1,0 +1,34 @@
+"""A fit queues its steps with overlapping launches: a step and its Adam update
+are on the GPU while the ones before still write the weights and partial sums
+that they read.  The same steps, one call each (and so each waited for), must
+give the same losses and weights bit for bit, at one, two and four CTAs per 128
+samples."""
+import numpy as np
+import pytest
+
+from paper_1010_1486_gb300 import learn, su2
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("batch,steps", [(128, 400), (4096, 400), (76 * 128, 200), (16384, 100), (65536, 40)])
+def test_overlapped_steps_equal_separate_ones(batch, steps):
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(batch)
+    n = 50_000
+    bk = np.clip(rng.normal(12.0, 3.0, n), 3.0, 30.0)
+    pairs = np.stack([bk, np.clip(1.0 - rng.gamma(1.5, size=n) / bk, -1.0, 1.0)], axis=1).astype(np.float32)
+    dev = torch.from_numpy(pairs).cuda()
+    out = []
+    for calls in ([steps], [1] * steps):
+        tr = su2.su2_trainer_create(learn.initial_weights(5), 9)
+        try:
+            su2.su2_trainer_set_input_scaling(tr, dev.data_ptr(), n)
+            losses = [su2.su2_trainer_fit(tr, dev.data_ptr(), n, k, batch) for k in calls]
+            out.append((np.concatenate(losses), su2.su2_trainer_get_weights(tr)))
+        finally:
+            su2.su2_trainer_destroy(tr)
+    (la, wa), (lb, wb) = out
+    assert np.array_equal(la.view(np.uint32), lb.view(np.uint32))
+    assert np.array_equal(wa.view(np.uint32), wb.view(np.uint32))
+    assert np.isfinite(la).all() and la[-5:].mean() < la[:5].mean()
