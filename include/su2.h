@@ -422,9 +422,14 @@ su2_status su2_batch_launch_info(su2_batch *b, int *queue_depth, int *threads, i
 su2_status su2_batch_autotune(su2_batch *b, int sweeps, int *queue_depth, int *grid);
 su2_status su2_batch_info(su2_batch *b, int *n, uint32_t *sweep, int *queue_depth, int *grid, int *graphs);
 
-/* Self-test of the bounded grid-barrier wait: `blocks` blocks wait for one
- * arrival more than there are blocks, so every wait must give up after
- * timeout_ns (<= 5 s); *timed_out receives the number of blocks that did. */
+/* Self-test of the batch's grid barrier, the function that the sweeps call:
+ * `blocks` blocks (1..1024) pass `barriers` barriers (0..1000) that complete,
+ * then wait for one arrival more than there are blocks, so that every wait
+ * must give up after timeout_ns (<= 5 s).  counts[0]: blocks whose wait gave
+ * up; counts[1]: writes of another block not seen after a barrier (0);
+ * counts[2]: the barrier's error word (1).  su2_selftest_barrier_timeout: the
+ * same without completing barriers, *timed_out = counts[0]. */
+su2_status su2_selftest_barrier(int blocks, int barriers, uint64_t timeout_ns, unsigned int *counts);
 su2_status su2_selftest_barrier_timeout(int blocks, uint64_t timeout_ns, unsigned int *timed_out);
 
 /* Self-test of the bounded mbarrier wait that the learned phase uses for its

@@ -22,29 +22,21 @@
 
 namespace su2 {
 
-// Self-test of the barrier's timeout: `expect` arrivals are awaited but only
-// gridDim.x blocks exist, so with expect > gridDim.x every wait must give up
-// after timeout_ns and report it.  The arrival count is reset for the next use.
-__global__ void barrier_timeout_kernel(BarrierState *bar, unsigned int expect, unsigned long long timeout_ns,
-                                       unsigned int *timed_out)
+// Self-test of grid_barrier: `barriers` barriers that complete, each block
+// publishing its number before and reading its neighbour's after, then one
+// that waits for one arrival more than there are blocks.  counts: [0] blocks
+// whose last wait gave up, [1] neighbours seen late.
+__global__ void barrier_selftest_kernel(BarrierState *bar, unsigned int barriers, unsigned long long timeout_ns,
+                                        unsigned int *seen, unsigned int *counts)
 {
-    if (threadIdx.x == 0) {
-        volatile unsigned int *vgen = &bar->gen;
-        const unsigned int g = *vgen;
-        const unsigned int arrived = atomicAdd(&bar->count, 1u) + 1u;
-        if (arrived == expect) {
-            atomicAdd(&bar->gen, 1u);
-        } else {
-            const unsigned long long t0 = global_time_ns();
-            while (*vgen == g) {
-                if (global_time_ns() - t0 > timeout_ns) {
-                    atomicAdd(timed_out, 1u);
-                    break;
-                }
-                __nanosleep(1000);
-            }
-        }
+    const unsigned int next = (blockIdx.x + 1u) % gridDim.x;
+    bool ok = true;
+    for (unsigned int b = 0; b < barriers && ok; ++b) {
+        if (threadIdx.x == 0) seen[blockIdx.x] = b + 1u;
+        ok = grid_barrier(bar, b, timeout_ns, gridDim.x);
+        if (ok && threadIdx.x == 0 && __ldcg(seen + next) < b + 1u) atomicAdd(&counts[1], 1u);
     }
+    if (ok && !grid_barrier(bar, barriers, timeout_ns, gridDim.x + 1u) && threadIdx.x == 0) atomicAdd(&counts[0], 1u);
 }
 
 }  // namespace su2
@@ -664,27 +656,37 @@ su2_status su2_batch_autotune(su2_batch *b, int sweeps, int *queue_depth, int *g
     return st;
 }
 
-su2_status su2_selftest_barrier_timeout(int blocks, uint64_t timeout_ns, unsigned int *timed_out)
+su2_status su2_selftest_barrier(int blocks, int barriers, uint64_t timeout_ns, unsigned int *counts)
 {
-    if (blocks < 1 || blocks > 1024 || !timed_out || timeout_ns > 5000000000ull) return SU2_E_INVAL;
+    constexpr int kMost = 1024;
+    if (blocks < 1 || blocks > kMost || barriers < 0 || barriers > 1000 || !counts || timeout_ns > 5000000000ull)
+        return SU2_E_INVAL;
     int dev = 0;
     SU2_CUDA(cudaGetDevice(&dev));
-    const size_t bytes = 256 + sizeof(unsigned int);
+    const size_t bytes = sizeof(BarrierState) + sizeof(unsigned int) * (kMost + 2);
     char *buf = (char *)device_alloc(bytes, dev, nullptr);
     if (!buf) return SU2_E_NOMEM;
-    su2_status st = SU2_OK;
     BarrierState *bar = (BarrierState *)buf;
-    unsigned int *count = (unsigned int *)(buf + 256);
-    if (cudaMemsetAsync(buf, 0, bytes, nullptr) != cudaSuccess) st = cuda_fail(cudaGetLastError(), "memset");
-    if (st == SU2_OK) {
-        // one more arrival is expected than there are blocks: nothing completes the barrier
-        barrier_timeout_kernel<<<blocks, 32>>>(bar, (unsigned int)blocks + 1u, timeout_ns, count);
-        cudaError_t e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaMemcpy(timed_out, count, sizeof(unsigned int), cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) st = cuda_fail(e, "barrier self-test");
-    }
+    unsigned int *seen = (unsigned int *)(bar + 1), *d_counts = seen + kMost;
+    unsigned int nbar = (unsigned int)barriers;
+    unsigned long long limit = timeout_ns;
+    void *args[] = {&bar, &nbar, &limit, &seen, &d_counts};
+    cudaError_t e = cudaMemsetAsync(buf, 0, bytes, nullptr);
+    if (e == cudaSuccess)
+        e = cudaLaunchCooperativeKernel((const void *)barrier_selftest_kernel, dim3(blocks), dim3(32), args, 0, nullptr);
+    if (e == cudaSuccess) e = cudaMemcpy(counts, d_counts, 2 * sizeof *counts, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(counts + 2, &bar->error, sizeof *counts, cudaMemcpyDeviceToHost);
     device_free(buf, bytes, dev, nullptr);
     cudaStreamSynchronize(nullptr);
+    return e == cudaSuccess ? SU2_OK : cuda_fail(e, "barrier self-test");
+}
+
+su2_status su2_selftest_barrier_timeout(int blocks, uint64_t timeout_ns, unsigned int *timed_out)
+{
+    unsigned int counts[3];
+    if (!timed_out) return SU2_E_INVAL;
+    const su2_status st = su2_selftest_barrier(blocks, 0, timeout_ns, counts);
+    if (st == SU2_OK) *timed_out = counts[0];
     return st;
 }
 

@@ -123,6 +123,7 @@ _SIGS = {
     "su2_batch_autotune": [_P, _i32, ctypes.POINTER(_i32), ctypes.POINTER(_i32)],
     "su2_batch_info": [_P, ctypes.POINTER(_i32), ctypes.POINTER(_u32), ctypes.POINTER(_i32), ctypes.POINTER(_i32),
                        ctypes.POINTER(_i32)],
+    "su2_selftest_barrier": [_i32, _i32, _u64, _P],
     "su2_selftest_barrier_timeout": [_i32, _u64, ctypes.POINTER(_u32)],
     "su2_selftest_mbar_timeout": [_i32, _u32, ctypes.POINTER(_u32)],
     "su2_selftest_mma": [_P, _P, _i32, _P],
@@ -659,6 +660,13 @@ def su2_batch_info(b: int) -> dict:
     _check(_lib.su2_batch_info(b, ctypes.byref(n), ctypes.byref(sw), ctypes.byref(r), ctypes.byref(g),
                                ctypes.byref(gr)), "su2_batch_info")
     return {"n": n.value, "sweep": sw.value, "queue_depth": r.value, "grid": g.value, "graphs": bool(gr.value)}
+
+
+def su2_selftest_barrier(blocks: int, barriers: int, timeout_ns: int) -> list:
+    """[blocks whose last wait gave up, stale reads after a barrier, error word]"""
+    counts = np.zeros(3, dtype=np.uint32)
+    _check(_lib.su2_selftest_barrier(blocks, barriers, timeout_ns, _host_ptr(counts)), "su2_selftest_barrier")
+    return counts.tolist()
 
 
 def su2_selftest_barrier_timeout(blocks: int, timeout_ns: int) -> int:
