@@ -432,6 +432,12 @@ su2_status su2_batch_info(su2_batch *b, int *n, uint32_t *sweep, int *queue_dept
 su2_status su2_selftest_barrier(int blocks, int barriers, uint64_t timeout_ns, unsigned int *counts);
 su2_status su2_selftest_barrier_timeout(int blocks, uint64_t timeout_ns, unsigned int *timed_out);
 
+/* Self-test of a batch call whose barrier wait gave up: as su2_batch_generate,
+ * with the error word set before the first sweep.  The sweeps queued behind it
+ * do nothing, and the call returns SU2_E_DEVICE_TIMEOUT; the next call starts
+ * with the word cleared. */
+su2_status su2_selftest_batch_stopped(su2_batch *b, int nsweeps, int measure_every, su2_stats *stats);
+
 /* Self-test of the bounded mbarrier wait that the learned phase uses for its
  * proposal-table copy: in each of `blocks` blocks (1..1024) thread 0 sets up
  * an mbarrier that expects one arrival which never comes, and waits `polls`

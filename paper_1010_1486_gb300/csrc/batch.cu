@@ -14,6 +14,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -66,7 +67,9 @@ struct su2_batch {
     int2 *d_poly_rounds = nullptr;       // [total_poly_rounds]
     int total_poly_rounds = 0;
     BarrierState *d_bar = nullptr;
-    unsigned int *d_counters = nullptr;  // [0] sweep, [1] measurement index, [2..] flags
+    // from the barrier's error word on: error, then d_flags [0] sampler failures, [1] hot-start failures, d_meas
+    // (measurement index), d_sweep.  A call clears all but the sweep.
+    unsigned int *d_flags = nullptr, *d_meas = nullptr, *d_sweep = nullptr;
     unsigned long long *d_trials = nullptr;
     double *d_history = nullptr;
     int history_cap = 0;
@@ -142,8 +145,8 @@ BatchParams params_of(const su2_batch *b, int do_sweep, int measure)
     p.total_poly_rounds = b->total_poly_rounds;
     p.do_sweep = do_sweep;
     p.measure = measure;
-    p.sweep = b->d_counters;
-    p.meas_index = b->d_counters + 1;
+    p.sweep = b->d_sweep;
+    p.meas_index = b->d_meas;
     p.round_partials = b->d_partials;
     p.fused = do_sweep && measure;
     p.chunk_partials = b->d_chunk_partials;
@@ -152,14 +155,16 @@ BatchParams params_of(const su2_batch *b, int do_sweep, int measure)
     p.bar = b->d_bar;
     p.timeout_ns = b->timeout_ns;
     p.trial_slots = b->d_trials;
-    p.flags = b->d_counters + 2;
+    p.flags = b->d_flags;
     return p;
 }
 
-// Enqueues one launch: reset of the barrier state, then the cooperative kernel.
+// Enqueues one launch: reset of the barrier's arrivals, then the cooperative
+// kernel.  The error word stays: a sweep that was given up is reported by the
+// call even if others were queued behind it, and those do nothing.
 cudaError_t enqueue_launch(su2_batch *b, int do_sweep, int measure)
 {
-    cudaError_t e = cudaMemsetAsync(b->d_bar, 0, sizeof(BarrierState), b->stream);
+    cudaError_t e = cudaMemsetAsync(b->d_bar, 0, offsetof(BarrierState, error), b->stream);
     if (e != cudaSuccess) return e;
     BatchParams p = params_of(b, do_sweep, measure);
     void *args[] = {&p};
@@ -204,9 +209,11 @@ su2_status launch_sweep(su2_batch *b, int measure)
 }
 
 // Places in the block from the barrier state on.
-constexpr size_t kCountersAt = 256, kTrialsAt = 512;
+constexpr size_t kCountersAt = sizeof(BarrierState), kTrialsAt = 512;
 constexpr size_t kCheckBytes = kTrialsAt + sizeof(unsigned long long) * 8 * kTrialSlots;
-static_assert(sizeof(BarrierState) <= kCountersAt, "the counters follow the barrier state");
+constexpr size_t kErrorAt = offsetof(BarrierState, error);
+static_assert(kErrorAt + sizeof(unsigned int) == kCountersAt, "error word, flags and measurement index are one range");
+constexpr size_t kClearBytes = 4 * sizeof(unsigned int);
 
 // Reads the batch's status (synchronises), through the first kCheckBytes of `page` if it has one.
 su2_status check_flags(su2_batch *b, su2_stats *stats, uint64_t sweeps, int launches, const HostPage &page)
@@ -228,27 +235,28 @@ su2_status check_flags(su2_batch *b, su2_stats *stats, uint64_t sweeps, int laun
             for (int j = 0; j < kTrialSlots; ++j) s += slots[ph * kTrialSlots + j];
             stats->trials[ph] = s;
         }
-        stats->sampler_failures = counters[2];
+        stats->sampler_failures = counters[0];
         stats->sweeps = sweeps;
         stats->link_updates = sweeps * 4ull * sites;
         stats->kernel_launches = (uint32_t)launches;
     }
-    b->sweep = counters[0];
+    b->sweep = counters[3];
     if (bar.error & 1u) {
         set_last_error("batch sweep: a grid barrier wait timed out");
         return SU2_E_DEVICE_TIMEOUT;
     }
-    if (counters[2]) {
+    if (counters[0]) {
         set_last_error("heat-bath sampler hit its trial cap");
         return SU2_E_SAMPLER;
     }
     return SU2_OK;
 }
 
+// Start of a call: trial counters, error word, flags and measurement index.
 su2_status clear_stats(su2_batch *b)
 {
     SU2_CUDA(cudaMemsetAsync(b->d_trials, 0, sizeof(unsigned long long) * 8 * kTrialSlots, b->stream));
-    SU2_CUDA(cudaMemsetAsync(b->d_counters + 2, 0, sizeof(unsigned int) * 2, b->stream));
+    SU2_CUDA(cudaMemsetAsync(&b->d_bar->error, 0, kClearBytes, b->stream));
     return SU2_OK;
 }
 
@@ -378,7 +386,9 @@ su2_status su2_batch_create(int n, const int *ns, const int *nt, const double *b
     p += align256(sizeof(int2) * poly_rounds.size());
     b->d_bar = (BarrierState *)p;
     p += bar_bytes;
-    b->d_counters = (unsigned int *)p;
+    b->d_flags = (unsigned int *)p;
+    b->d_meas = b->d_flags + 2;
+    b->d_sweep = b->d_flags + 3;
     p += counter_bytes;
     b->d_trials = (unsigned long long *)p;
 
@@ -405,8 +415,8 @@ su2_status su2_batch_create(int n, const int *ns, const int *nt, const double *b
                             cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_bar, 0, bar_bytes + counter_bytes + trial_bytes, b->stream);
     for (int l = 0; l < n && e == cudaSuccess; ++l)
-        e = start_links(b->links + b->link_offset[l], b->geom[l], start == SU2_HOT, seed[l], b->d_counters + 2,
-                        b->stream);  // the hot-start kernel counts failures in flags[1] = counter 3
+        e = start_links(b->links + b->link_offset[l], b->geom[l], start == SU2_HOT, seed[l], b->d_flags,
+                        b->stream);  // the hot-start kernel counts failures in flags[1]
     if (e == cudaSuccess) {
         int sms = 0;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -423,11 +433,11 @@ su2_status su2_batch_create(int n, const int *ns, const int *nt, const double *b
     if (e != cudaSuccess) st = cuda_fail(e, "su2_batch_create");
     if (st == SU2_OK) st = set_depth(b, 4, 128, b->max_grid[0][r_index(4)][t_index(128)]);
     if (st == SU2_OK) {
-        unsigned int c[4];
-        if (cudaMemcpyAsync(c, b->d_counters, sizeof c, cudaMemcpyDeviceToHost, b->stream) != cudaSuccess ||
+        unsigned int c[2];
+        if (cudaMemcpyAsync(c, b->d_flags, sizeof c, cudaMemcpyDeviceToHost, b->stream) != cudaSuccess ||
             cudaStreamSynchronize(b->stream) != cudaSuccess)
             st = cuda_fail(cudaGetLastError(), "su2_batch_create");
-        else if (c[3]) {
+        else if (c[1]) {
             set_last_error("hot start: a link found no two disk points in 64 pairs");
             st = SU2_E_SAMPLER;
         }
@@ -455,8 +465,9 @@ su2_status su2_batch_destroy(su2_batch *b)
     return SU2_OK;
 }
 
-su2_status su2_batch_generate(su2_batch *b, int nsweeps, int measure_every, double *plaq, double *poly,
-                              su2_stats *stats)
+// su2_batch_generate; stopped: the error word is set before the first sweep (self-test).
+static su2_status batch_generate(su2_batch *b, int nsweeps, int measure_every, double *plaq, double *poly,
+                                 su2_stats *stats, bool stopped)
 {
     if (!b || nsweeps < 0 || measure_every < 0) return SU2_E_INVAL;
     DeviceGuard guard(b->device);
@@ -464,7 +475,7 @@ su2_status su2_batch_generate(su2_batch *b, int nsweeps, int measure_every, doub
     su2_status st = ensure_history(b, std::max(nmeas, 1));
     if (st != SU2_OK) return st;
     if ((st = clear_stats(b)) != SU2_OK) return st;
-    SU2_CUDA(cudaMemsetAsync(b->d_counters + 1, 0, sizeof(unsigned int), b->stream));
+    if (stopped) SU2_CUDA(cudaMemsetAsync(&b->d_bar->error, 1, 1, b->stream));
     for (int s = 1; s <= nsweeps; ++s) {
         const int measure = (measure_every > 0 && s % measure_every == 0) ? 1 : 0;
         if ((st = launch_sweep(b, measure)) != SU2_OK) return st;
@@ -490,6 +501,17 @@ su2_status su2_batch_generate(su2_batch *b, int nsweeps, int measure_every, doub
     return st;
 }
 
+su2_status su2_batch_generate(su2_batch *b, int nsweeps, int measure_every, double *plaq, double *poly,
+                              su2_stats *stats)
+{
+    return batch_generate(b, nsweeps, measure_every, plaq, poly, stats, false);
+}
+
+su2_status su2_selftest_batch_stopped(su2_batch *b, int nsweeps, int measure_every, su2_stats *stats)
+{
+    return batch_generate(b, nsweeps, measure_every, nullptr, nullptr, stats, true);
+}
+
 su2_status su2_batch_sweep(su2_batch *b, int nsweeps, su2_stats *stats)
 {
     return su2_batch_generate(b, nsweeps, 0, nullptr, nullptr, stats);
@@ -501,7 +523,7 @@ su2_status su2_batch_measure(su2_batch *b, double *plaq, double *poly)
     DeviceGuard guard(b->device);
     su2_status st = ensure_history(b, 1);
     if (st != SU2_OK) return st;
-    SU2_CUDA(cudaMemsetAsync(b->d_counters + 1, 0, sizeof(unsigned int), b->stream));
+    SU2_CUDA(cudaMemsetAsync(&b->d_bar->error, 0, kClearBytes, b->stream));
     SU2_CUDA(enqueue_launch(b, 0, 1));
     std::vector<double> h(2 * (size_t)b->n);
     SU2_CUDA(cudaMemcpyAsync(h.data(), b->d_history, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, b->stream));
@@ -612,6 +634,7 @@ su2_status su2_batch_autotune(su2_batch *b, int sweeps, int *queue_depth, int *g
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess ||
         cudaMemcpyAsync(saved, b->links, bytes, cudaMemcpyDeviceToDevice, b->stream) != cudaSuccess)
         st = cuda_fail(cudaGetLastError(), "su2_batch_autotune");
+    if (st == SU2_OK) st = clear_stats(b);
     const int depths[4] = {1, 2, 4, 8};
     for (int c = 0; c < kAutotuneCandidates && st == SU2_OK; ++c) {
             const int i = c / (3 * kGridFractions), j = (c / kGridFractions) % 3, f = c % kGridFractions;
@@ -627,9 +650,19 @@ su2_status su2_batch_autotune(su2_batch *b, int sweeps, int *queue_depth, int *g
                 st = cuda_fail(cudaGetLastError(), "su2_batch_autotune");
                 break;
             }
+            // a launch behind one that was given up does nothing: no candidate may win that way
+            unsigned int error = 0;
+            if (cudaMemcpyAsync(&error, &b->d_bar->error, sizeof error, cudaMemcpyDeviceToHost, b->stream) !=
+                    cudaSuccess ||
+                cudaStreamSynchronize(b->stream) != cudaSuccess)
+                st = cuda_fail(cudaGetLastError(), "su2_batch_autotune");
+            else if (error & 1u) {
+                set_last_error("batch autotuning: a grid barrier wait timed out");
+                st = SU2_E_DEVICE_TIMEOUT;
+            }
             float ms = 0.0f;
             cudaEventElapsedTime(&ms, e0, e1);
-            if (ms < best) {
+            if (st == SU2_OK && ms < best) {
                 best = ms;
                 best_r = R;
                 best_t = T;
@@ -637,7 +670,7 @@ su2_status su2_batch_autotune(su2_batch *b, int sweeps, int *queue_depth, int *g
             }
             // restore the configuration the candidates started from
             if (cudaMemcpyAsync(b->links, saved, bytes, cudaMemcpyDeviceToDevice, b->stream) != cudaSuccess ||
-                cudaMemcpyAsync(b->d_counters, &sweep0, sizeof sweep0, cudaMemcpyHostToDevice, b->stream) !=
+                cudaMemcpyAsync(b->d_sweep, &sweep0, sizeof sweep0, cudaMemcpyHostToDevice, b->stream) !=
                     cudaSuccess ||
                 cudaStreamSynchronize(b->stream) != cudaSuccess) {
                 st = cuda_fail(cudaGetLastError(), "su2_batch_autotune");

@@ -31,12 +31,13 @@ struct LatDesc {
 };
 
 // Arrivals and release on lines of their own: the polls of the waiting blocks
-// do not slow the atomics of the arriving ones.  Zeroed before every launch;
-// both numbers only grow during it.
+// do not slow the atomics of the arriving ones.  Zeroed before every launch but
+// for the error word; both numbers only grow during it.
 struct BarrierState {
     alignas(128) unsigned int count;  // arrivals
     alignas(128) unsigned int gen;    // barriers completed
-    unsigned int error;               // bit 0: a barrier wait timed out
+    unsigned int pad[30];
+    unsigned int error;               // bit 0: a barrier wait timed out; cleared at the start of a call
 };
 
 struct BatchParams {
@@ -408,6 +409,7 @@ __global__ void __launch_bounds__(T, kBatchThreadsPerSm / T) batch_sweep_kernel(
     const int wib = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int warp_global = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (*(volatile unsigned int *)&bp.bar->error & 1u) return;  // an earlier launch of the call was given up
     const uint32_t sweep = *(volatile unsigned int *)bp.sweep;
     const unsigned int slot = *(volatile unsigned int *)bp.meas_index;
     const bool fused = bp.fused && (int)slot < bp.history_cap;

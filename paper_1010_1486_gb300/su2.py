@@ -112,6 +112,7 @@ _SIGS = {
     "su2_batch_create": [_i32, _P, _P, _P, _P, _i32, _P, ctypes.POINTER(_P)],
     "su2_batch_destroy": [_P],
     "su2_batch_sweep": [_P, _i32, ctypes.POINTER(su2_stats)],
+    "su2_selftest_batch_stopped": [_P, _i32, _i32, ctypes.POINTER(su2_stats)],
     "su2_batch_generate": [_P, _i32, _i32, _P, _P, ctypes.POINTER(su2_stats)],
     "su2_batch_plaquette": [_P, _P],
     "su2_batch_polyakov": [_P, _P],
@@ -660,6 +661,10 @@ def su2_batch_info(b: int) -> dict:
     _check(_lib.su2_batch_info(b, ctypes.byref(n), ctypes.byref(sw), ctypes.byref(r), ctypes.byref(g),
                                ctypes.byref(gr)), "su2_batch_info")
     return {"n": n.value, "sweep": sw.value, "queue_depth": r.value, "grid": g.value, "graphs": bool(gr.value)}
+
+
+def su2_selftest_batch_stopped(b: int, nsweeps: int, measure_every: int = 0) -> None:
+    _check(_lib.su2_selftest_batch_stopped(b, nsweeps, measure_every, None), "su2_selftest_batch_stopped")
 
 
 def su2_selftest_barrier(blocks: int, barriers: int, timeout_ns: int) -> list:
