@@ -216,13 +216,14 @@ static_assert(kErrorAt + sizeof(unsigned int) == kCountersAt, "error word, flags
 constexpr size_t kClearBytes = 4 * sizeof(unsigned int);
 
 // Reads the batch's status (synchronises), through the first kCheckBytes of `page` if it has one.
-su2_status check_flags(su2_batch *b, su2_stats *stats, uint64_t sweeps, int launches, const HostPage &page)
+su2_status check_flags(su2_batch *b, su2_stats *stats, uint64_t sweeps, int launches, HostPage &page)
 {
     // barrier state, counters and trial counters lie side by side: one copy
     alignas(128) char own[kCheckBytes];
     char *const to = page.p ? page.p : own;
     SU2_CUDA(cudaMemcpyAsync(to, b->d_bar, kCheckBytes, cudaMemcpyDeviceToHost, b->stream));
     SU2_CUDA(cudaStreamSynchronize(b->stream));
+    page.settled();
     const BarrierState &bar = *(const BarrierState *)to;
     const unsigned int *const counters = (const unsigned int *)(to + kCountersAt);
     const unsigned long long *const slots = (const unsigned long long *)(to + kTrialsAt);
@@ -480,7 +481,7 @@ static su2_status batch_generate(su2_batch *b, int nsweeps, int measure_every, d
         const int measure = (measure_every > 0 && s % measure_every == 0) ? 1 : 0;
         if ((st = launch_sweep(b, measure)) != SU2_OK) return st;
     }
-    const HostPage page;
+    HostPage page(b->stream);
     const size_t values = nmeas > 0 && (plaq || poly) ? (size_t)nmeas * 2 * b->n : 0;
     std::vector<double> own;
     double *h = (double *)(page.p + kCheckBytes);

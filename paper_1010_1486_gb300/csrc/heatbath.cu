@@ -643,15 +643,13 @@ su2_status su2_generate(su2_lattice *lat, int nsweeps, int measure_every, int re
 {
     if (!lat || nsweeps < 0 || measure_every < 0 || reunit_every < 0) return SU2_E_INVAL;
     DeviceGuard guard(lat->device);
-    const HostPage page;
+    HostPage page(lat->stream);
     ResultCopy copy(page, kStatsBytes, measure_every > 0 ? nsweeps / measure_every : 0, plaq, poly);
     su2_status st = generate_enqueue(lat, nsweeps, measure_every, reunit_every, copy.plaq, copy.poly, true);
-    if (st != SU2_OK) {
-        cudaStreamSynchronize(lat->stream);  // nothing may still be on its way to the page
-        return st;
-    }
+    if (st != SU2_OK) return st;
     if (stats) memset(stats, 0, sizeof *stats);
     st = collect_stats(lat, stats, (uint64_t)nsweeps, page);
+    if (st == SU2_E_CUDA) return st;  // the copies may not have arrived
     copy.finish();
     if (stats) {
         stats->kernel_launches = (uint32_t)(8 * nsweeps);

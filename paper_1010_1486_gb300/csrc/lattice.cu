@@ -65,49 +65,6 @@ void device_free(void *ptr, size_t bytes, int device, cudaStream_t stream)
     cudaFreeAsync(ptr, stream);
 }
 
-// ------------------------------------------------- page-locked result pages
-static std::mutex g_page_mutex;
-static char *g_pages[kHostPages];  // the free ones
-static int g_pages_free = 0, g_pages_made = 0, g_page_users = 0;
-
-HostPage::HostPage() : p(nullptr)
-{
-    std::lock_guard<std::mutex> lock(g_page_mutex);
-    if (g_pages_free > 0) {
-        p = g_pages[--g_pages_free];
-    } else if (g_pages_made < kHostPages) {
-        void *q = nullptr;
-        if (cudaHostAlloc(&q, kHostPageBytes, cudaHostAllocPortable) == cudaSuccess) {
-            p = (char *)q;
-            ++g_pages_made;
-        } else {
-            cudaGetLastError();
-        }
-    }
-}
-
-HostPage::~HostPage()
-{
-    if (!p) return;
-    std::lock_guard<std::mutex> lock(g_page_mutex);
-    g_pages[g_pages_free++] = p;
-}
-
-void host_pages_retain()
-{
-    std::lock_guard<std::mutex> lock(g_page_mutex);
-    ++g_page_users;
-}
-
-void host_pages_release()
-{
-    std::lock_guard<std::mutex> lock(g_page_mutex);
-    if (--g_page_users > 0) return;
-    g_pages_made -= g_pages_free;
-    while (g_pages_free > 0) cudaFreeHost(g_pages[--g_pages_free]);
-    cudaGetLastError();
-}
-
 // ------------------------------------------------------------- kernels
 __global__ void cold_start_kernel(float4 *__restrict__ links, int64_t n)
 {
@@ -218,12 +175,13 @@ su2_status launch_clear_counters(su2_lattice *lat)
     return SU2_OK;
 }
 
-su2_status collect_stats(su2_lattice *lat, su2_stats *stats, uint64_t sweeps, const HostPage &page)
+su2_status collect_stats(su2_lattice *lat, su2_stats *stats, uint64_t sweeps, HostPage &page)
 {
     alignas(8) char own[kStatsBytes];
     char *const to = page.p ? page.p : own;
     SU2_CUDA(cudaMemcpyAsync(to, lat->scratch.trials, kStatsBytes, cudaMemcpyDeviceToHost, lat->stream));
     SU2_CUDA(cudaStreamSynchronize(lat->stream));
+    page.settled();
     const unsigned long long *const slots = (const unsigned long long *)to;
     const unsigned int *const flags = (const unsigned int *)(slots + 8 * kTrialSlots);
     if (stats) {
@@ -549,11 +507,12 @@ su2_status su2_sync(su2_lattice *lat)
 {
     if (!lat) return SU2_E_INVAL;
     DeviceGuard guard(lat->device);
-    const HostPage page;
+    HostPage page(lat->stream);
     unsigned int own[4];
     unsigned int *const flags = page.p ? (unsigned int *)page.p : own;
     SU2_CUDA(cudaMemcpyAsync(flags, lat->scratch.flags, sizeof own, cudaMemcpyDeviceToHost, lat->stream));
     SU2_CUDA(cudaStreamSynchronize(lat->stream));
+    page.settled();
     if (flags[0] != 0) {
         SU2_CUDA(cudaMemsetAsync(lat->scratch.flags, 0, sizeof(unsigned int), lat->stream));
         SU2_CUDA(cudaStreamSynchronize(lat->stream));
@@ -568,7 +527,7 @@ su2_status su2_check_links(su2_lattice *lat, double tol, uint64_t *nonfinite, ui
     if (!lat || !(tol >= 0.0)) return SU2_E_INVAL;
     DeviceGuard guard(lat->device);
     unsigned long long *const d = (unsigned long long *)(lat->scratch.result + 2);
-    const HostPage page;
+    HostPage page(lat->stream);
     unsigned long long own[2];
     unsigned long long *const h = page.p ? (unsigned long long *)page.p : own;
     SU2_CUDA(cudaMemsetAsync(d, 0, sizeof own, lat->stream));
@@ -577,6 +536,7 @@ su2_status su2_check_links(su2_lattice *lat, double tol, uint64_t *nonfinite, ui
     SU2_CUDA(cudaGetLastError());
     SU2_CUDA(cudaMemcpyAsync(h, d, sizeof own, cudaMemcpyDeviceToHost, lat->stream));
     SU2_CUDA(cudaStreamSynchronize(lat->stream));
+    page.settled();
     if (nonfinite) *nonfinite = h[0];
     if (off_norm) *off_norm = h[1];
     if (h[0]) {

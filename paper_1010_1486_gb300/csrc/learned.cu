@@ -590,7 +590,7 @@ su2_status su2_learned_generate(su2_lattice *lat, int nsweeps, int measure_every
     }
     // the trial counters, the acceptance counters and control words (one copy:
     // they lie side by side), then the measurements
-    const HostPage page;
+    HostPage page(lat->stream);
     const size_t accept_at = kStatsBytes, accept_bytes = 256 + sizeof(unsigned long long) * 8 * kAcceptSlots;
     alignas(8) char own[accept_bytes];
     char *const to = page.p ? page.p + accept_at : own;
@@ -606,6 +606,7 @@ su2_status su2_learned_generate(su2_lattice *lat, int nsweeps, int measure_every
     su2_stats plain;
     memset(&plain, 0, sizeof plain);
     st = collect_stats(lat, &plain, (uint64_t)nsweeps, page);
+    if (st == SU2_E_CUDA) return st;  // the copies may not have arrived
     copy.finish();
     const unsigned int *const ctl = (const unsigned int *)to;
     const unsigned long long *const slots = (const unsigned long long *)(to + 256);

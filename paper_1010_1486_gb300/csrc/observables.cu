@@ -269,11 +269,12 @@ using namespace su2;
 // into a page-locked page itself, or, when none is free, to *dev to be copied.
 static su2_status read_value(su2_lattice *lat, su2_status (*launch)(su2_lattice *, double *), double *dev, double *out)
 {
-    const HostPage page;
+    HostPage page(lat->stream);
     su2_status st = launch(lat, page.p ? (double *)page.p : dev);
     if (st != SU2_OK) return st;
     if (!page.p) SU2_CUDA(cudaMemcpyAsync(out, dev, sizeof(double), cudaMemcpyDeviceToHost, lat->stream));
     SU2_CUDA(cudaStreamSynchronize(lat->stream));
+    page.settled();
     if (page.p) *out = *(const double *)page.p;
     return SU2_OK;
 }

@@ -260,7 +260,8 @@ su2_status su2_slab_stats(su2_slab *s, uint64_t trials[8], uint64_t *sampler_fai
     if (!s || !trials) return SU2_E_INVAL;
     DeviceGuard guard(s->lat->device);
     su2_stats st;
-    su2_status r = collect_stats(s->lat, &st, 0, HostPage());
+    HostPage page(s->lat->stream);
+    su2_status r = collect_stats(s->lat, &st, 0, page);
     // the kernels count by local parity; report by the global one
     for (int mu = 0; mu < 4; ++mu)
         for (int p = 0; p < 2; ++p) trials[2 * mu + p] = st.trials[2 * mu + local_parity(p)];

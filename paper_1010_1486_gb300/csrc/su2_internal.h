@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/su2.h"
+#include "host_pages.h"
 #include "su2_device.cuh"
 
 namespace su2 {
@@ -120,27 +121,6 @@ su2_status cuda_fail(cudaError_t e, const char *what);
         cudaError_t e_ = (call);                                               \
         if (e_ != cudaSuccess) return ::su2::cuda_fail(e_, #call);             \
     } while (0)
-
-// A page of page-locked host memory for the results of a synchronous call:
-// copies to it are queued behind the kernels, where a copy to pageable memory
-// waits for them (about 8 us each, one after the other).  Pages come from a
-// process-wide pool of at most kHostPages, taken for the duration of a call;
-// p is NULL when none is free (or page-locking failed), and the call then
-// copies to its caller's memory directly.
-constexpr size_t kHostPageBytes = 64 * 1024;
-constexpr int kHostPages = 16;
-struct HostPage {
-    char *p;
-    HostPage();
-    ~HostPage();
-    HostPage(const HostPage &) = delete;
-    HostPage &operator=(const HostPage &) = delete;
-};
-
-// Every lattice and batch retains the pages while it lives; the last one to go
-// gives them back.
-void host_pages_retain();
-void host_pages_release();
 
 // The two measurement histories of a call: their device copies go to plaq and
 // poly here -- behind the first `used` bytes of the page if they fit, else the
@@ -288,6 +268,6 @@ su2_status overrelax_sweeps(su2_lattice *lat, int n);
 // Reads the trial counters and flags (synchronises), through the first
 // kStatsBytes of `page` if it has one.
 constexpr size_t kStatsBytes = 8 * kTrialSlots * sizeof(unsigned long long) + 4 * sizeof(unsigned int);
-su2_status collect_stats(su2_lattice *lat, su2_stats *stats, uint64_t sweeps, const HostPage &page);
+su2_status collect_stats(su2_lattice *lat, su2_stats *stats, uint64_t sweeps, HostPage &page);
 
 }  // namespace su2

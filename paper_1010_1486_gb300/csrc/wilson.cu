@@ -458,13 +458,14 @@ extern "C" su2_status su2_wilson_loops(su2_lattice *lat, int rmax, int tmax, dou
     DeviceGuard guard(lat->device);
     const size_t n_out = (size_t)rmax * (size_t)tmax;
     const size_t bytes = sizeof(double) * n_out;
-    const HostPage page;
+    HostPage page(lat->stream);
     double own[kWilsonMaxR * kWilsonMaxT + 1];
     double *const host = page.p ? (double *)page.p : own;
     double *d_tiles = nullptr;
     SU2_CUDA(launch_tiles(lat, rmax, tmax, &d_tiles));
     SU2_CUDA(cudaMemcpyAsync(host, d_tiles, bytes + sizeof(double), cudaMemcpyDeviceToHost, lat->stream));
     SU2_CUDA(cudaStreamSynchronize(lat->stream));
+    page.settled();
     if (host[n_out] == 0.0) {
         std::copy(host, host + n_out, out);
         return SU2_OK;
