@@ -37,15 +37,25 @@ HostPage::~HostPage()
 void host_pages_retain()
 {
     std::lock_guard<std::mutex> lock(g_page_mutex);
-    ++g_page_users;
+    if (++g_page_users > 1) return;
+    // the pages kept while there was no handle: still there unless the program reset the device
+    for (int i = g_pages_free; i-- > 0;) {
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, g_pages[i]) == cudaSuccess && at.type == cudaMemoryTypeHost) continue;
+        g_pages[i] = g_pages[--g_pages_free];
+        --g_pages_made;
+    }
+    cudaGetLastError();
 }
 
 void host_pages_release()
 {
     std::lock_guard<std::mutex> lock(g_page_mutex);
     if (--g_page_users > 0) return;
-    g_pages_made -= g_pages_free;
-    while (g_pages_free > 0) cudaFreeHost(g_pages[--g_pages_free]);
+    while (g_pages_free > kHostPagesKept) {
+        cudaFreeHost(g_pages[--g_pages_free]);
+        --g_pages_made;
+    }
     cudaGetLastError();
 }
 

@@ -32,7 +32,11 @@ private:
 };
 
 // Every lattice and batch retains the pages while it lives; the last one to go
-// gives them back.
+// gives them back but for kHostPagesKept, which stays with the process.  A
+// program that makes a lattice, reads a value and destroys it, again and again,
+// would otherwise page-lock and free a page each time: 8^4, us per such turn
+// 211 without pages, 542 with all of them given back, 197 so.
+constexpr int kHostPagesKept = 1;
 void host_pages_retain();
 void host_pages_release();
 

@@ -25,6 +25,11 @@ cudaError_t cudaFreeHost(void *p)
     free(p);
     return cudaSuccess;
 }
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *at, const void *)
+{
+    at->type = live > 0 ? cudaMemoryTypeHost : cudaMemoryTypeUnregistered;
+    return cudaSuccess;
+}
 cudaError_t cudaStreamSynchronize(cudaStream_t s)
 {
     ++n_sync;
@@ -61,6 +66,25 @@ int main(int argc, char **argv)
         }
         host_pages_release();
         printf("%d\n", n_alloc);
+    }
+    if (!strcmp(what, "turns")) {
+        for (int turn = 0; turn < 5; ++turn) {
+            host_pages_retain();
+            HostPage *p[3];
+            for (HostPage *&q : p) (q = new HostPage(a))->settled();
+            for (HostPage *q : p) delete q;
+            host_pages_release();
+        }
+        printf("%d %d %d ", n_alloc, n_free, live);
+        live = 0;  // the program resets the device: the page kept is gone
+        host_pages_retain();
+        {
+            HostPage p(a);
+            p.settled();
+        }
+        printf("%d %d ", n_alloc, n_free);
+        host_pages_release();
+        printf("%d %d\n", n_free, live);
     }
     return 0;
 }

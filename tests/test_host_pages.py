@@ -31,3 +31,10 @@ def test_a_call_that_returns_early_waits_for_its_stream(scenario):
     # no wait after settled(); one on the page's own stream without; the pool
     # holds 16 pages, and a call without a page has nothing to wait for
     assert scenario("settle") == [0, 1, 1, 1, 16, 16]
+
+
+def test_one_page_stays_when_the_last_handle_goes(scenario):
+    """Five turns of a handle with three pages: the first makes three, the
+    others two each, and two go back at the end of each.  A page that a device
+    reset took away is forgotten, not freed, and a new one made."""
+    assert scenario("turns") == [3 + 4 * 2, 5 * 2, 1, 12, 10, 10, 1]
