@@ -280,6 +280,11 @@ __global__ void __launch_bounds__(kLearnThreads) collect_kernel(const float4 *__
     pairs[q] = make_float2(d.bk, a0);
 }
 
+constexpr int kMaxGridPoints = 400;  // rows of a proposal table
+// Bytes of the row pairs of a G-row table, rounded up to 16 (a bulk copy
+// moves a multiple of 16 bytes).
+static size_t pair_bytes_of(int G) { return (sizeof(float2) * (size_t)(G - 1) * learned::kParams + 15) & ~(size_t)15; }
+
 // Grid of all co-resident blocks (at most `want`), for the kernels that walk
 // their links in a loop.
 template <typename Kernel>
@@ -287,7 +292,9 @@ static cudaError_t launch_persistent(Kernel kernel, const LearnedParams &p, int 
                                      su2_lattice *lat)
 {
     int per_sm = 0, sms = 0;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit belongs to the kernel, which other threads launch too: always that of the largest table
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)pair_bytes_of(kMaxGridPoints));
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kLearnThreads, smem);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, lat->device);
     if (e != cudaSuccess) return e;
@@ -296,10 +303,6 @@ static cudaError_t launch_persistent(Kernel kernel, const LearnedParams &p, int 
     kernel<<<grid, kLearnThreads, smem, lat->stream>>>(p);
     return cudaGetLastError();
 }
-
-// Bytes of the row pairs of a G-row table, rounded up to 16 (a bulk copy
-// moves a multiple of 16 bytes).
-static size_t pair_bytes_of(int G) { return (sizeof(float2) * (size_t)(G - 1) * learned::kParams + 15) & ~(size_t)15; }
 
 static su2_status launch_learned_phase(su2_lattice *lat, int mu, int parity)
 {
@@ -457,7 +460,7 @@ extern "C" {
 
 su2_status su2_set_proposal(su2_lattice *lat, const float *weights, int n, double s_lo, double s_hi, int grid_points)
 {
-    if (!lat || !weights || n != learned::kWeights || grid_points < 2 || grid_points > 400 || !(s_hi > s_lo) ||
+    if (!lat || !weights || n != learned::kWeights || grid_points < 2 || grid_points > kMaxGridPoints || !(s_hi > s_lo) ||
         !std::isfinite(s_lo) || !std::isfinite(s_hi)) {
         set_last_error("su2_set_proposal: 1947 weights, 2 <= grid_points <= 400, finite s_lo < s_hi");
         return SU2_E_INVAL;
@@ -468,11 +471,11 @@ su2_status su2_set_proposal(su2_lattice *lat, const float *weights, int n, doubl
             return SU2_E_NUMERIC;
         }
     DeviceGuard guard(lat->device);
-    const size_t table_bytes = align256(sizeof(float) * learned::kParams * 400);
+    const size_t table_bytes = align256(sizeof(float) * learned::kParams * kMaxGridPoints);
     const size_t w_bytes = align256(sizeof(float) * learned::kWeights);
     const size_t ctl_bytes = align256(sizeof(unsigned int) * 4);
     const size_t slot_bytes = align256(sizeof(unsigned long long) * 9 * kAcceptSlots);
-    const size_t pairs_bytes = align256(pair_bytes_of(400));
+    const size_t pairs_bytes = align256(pair_bytes_of(kMaxGridPoints));
     if (!lat->learned_block) {
         lat->learned_bytes = table_bytes + w_bytes + ctl_bytes + slot_bytes + pairs_bytes;
         lat->learned_block = device_alloc(lat->learned_bytes, lat->device, lat->stream);

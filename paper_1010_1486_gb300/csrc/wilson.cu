@@ -68,9 +68,9 @@ struct TileSmem {
     int ucols, ut, s, total;
 };
 
-__host__ __device__ inline TileSmem tile_smem(int bx, int bt, int ns, int r0)
+__host__ __device__ constexpr TileSmem tile_smem(int bx, int bt, int ns, int r0)
 {
-    TileSmem m;
+    TileSmem m = {};
     m.ucols = bx + r0 + kLoopChunk < ns ? bx + r0 + kLoopChunk : ns;
     const int buf = 2 * bt * (bx + kLoopChunk), ui = (bt + kLoopChunk) * m.ucols;
     m.ut = buf > ui ? buf : ui;
@@ -78,6 +78,12 @@ __host__ __device__ inline TileSmem tile_smem(int bx, int bt, int ns, int r0)
     m.total = m.s + kTopPitch * (bt + kLoopChunk) * bx;
     return m;
 }
+
+// The most that a tile takes: kTileMaxBx columns of a longer row, the second
+// chunk of R.  (Narrower tiles have more rows, but at most 256 sites all the
+// same, and their staged rows end at the extent.)
+constexpr size_t kTileMaxSmem =
+    sizeof(float4) * (size_t)tile_smem(kTileMaxBx, kTileThreads / kTileMaxBx, 1 << 20, kWilsonMaxR - kLoopChunk).total;
 
 // FULL: the chunk has all eight R (no test per R in the inner loop).
 template <bool FULL>
@@ -425,7 +431,9 @@ static cudaError_t launch_tiles(su2_lattice *lat, int rmax, int tmax, double **d
     if (e != cudaSuccess) return e;
     const size_t smem = sizeof(float4) * (size_t)tile_smem(tl.bx, tl.bt, g.ns, (tl.nr - 1) * kLoopChunk).total;
     const auto kernel = rmax % kLoopChunk == 0 ? wilson_tile_kernel<true> : wilson_tile_kernel<false>;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit belongs to the kernel, which other threads launch too: always the most that a tile takes
+    e = smem <= kTileMaxSmem ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileMaxSmem)
+                             : cudaErrorInvalidValue;
     if (e != cudaSuccess) return e;
     const unsigned int blocks = 3u * (unsigned int)(g.ns * g.ns) * (unsigned int)(tl.nx * tl.nt * tl.nr * tl.ntc);
     const int threads = std::max(32, (tl.bx * tl.bt + 31) & ~31);
