@@ -6,8 +6,8 @@
 //   A = S_R(x) T_T(x+Ri),  B = T_T(x) S_R(x+Tt),  loop = (1/2) Tr A B^dag = A . B,
 // line products left to right, binary32 per loop (the link-arithmetic
 // contract); the mean over x and i = 0, 1, 2 is exact to 2^-44 per loop in
-// fixed point (wilson_tile_kernel), or binary64 for configurations whose loops
-// leave the fixed-point range (wilson_kernel).
+// fixed point (wilson_tile_kernel), or binary64 (wilson_kernel) for few small
+// loops, and for configurations whose loops leave the fixed-point range.
 #include <algorithm>
 
 #include "observables.cuh"
@@ -51,31 +51,36 @@ constexpr int kTileThreads = 256;      // most sites of a tile
 constexpr int kTileMaxBx = 64;         // most columns of a tile
 constexpr float kSplit = 6.0f;         // its neighbours lie 2^-21 apart
 constexpr unsigned int kSplitBits = 0x40C00000u;
-constexpr int kTopPitch = kLoopChunk + 1;  // float4 per site of s_buf: an odd pitch keeps 16-byte reads conflict-free
 
 struct LoopTiles {
     int bx, bt;          // tile extents along i and t
+    int rc, tc;          // most extents R and T of a chunk of this call
     int nx, nt, nr, ntc;  // tiles along i, along t, chunks of R, chunks of T
 };
 
 __device__ __forceinline__ int wrap_once(int c, int extent) { return c >= extent ? c - extent : c; }
 
-// Shared memory of a tile with extents bx x bt, in float4: [0] the two T_T
-// buffers, which first hold the staged U_i (rows t0 + tc0 .. + bt + 8, columns
-// x0 .. x0 + ucols - 1, all of them when they cover the extent), [1] the staged
-// U_t (rows t0 + tc0 .. + bt + 7), [2] s_buf.
+// Shared memory of a tile with extents bx x bt for chunks of up to rc x tc
+// extents, in float4: [0] the two T_T buffers, which first hold the staged U_i
+// (rows t0 + tc0 .. + bt + tc - 1, columns x0 .. x0 + ucols - 1, all of them when
+// they cover the extent), [1] the staged U_t (one row less), [2] s_buf.  (Laid
+// out for 8 x 8 extents whatever the call asked for, a tile of 56 columns left
+// room for one block per SM: 56^4, R = T = 1, 3.3 ms instead of 1.3.)
 struct TileSmem {
     int ucols, ut, s, total;
 };
 
-__host__ __device__ constexpr TileSmem tile_smem(int bx, int bt, int ns, int r0)
+// float4 per site of s_buf: an odd pitch keeps 16-byte reads conflict-free
+__host__ __device__ constexpr int top_pitch(int rc) { return rc | 1; }
+
+__host__ __device__ constexpr TileSmem tile_smem(int bx, int bt, int rc, int tc, int ns, int r0)
 {
     TileSmem m = {};
-    m.ucols = bx + r0 + kLoopChunk < ns ? bx + r0 + kLoopChunk : ns;
-    const int buf = 2 * bt * (bx + kLoopChunk), ui = (bt + kLoopChunk) * m.ucols;
+    m.ucols = bx + r0 + rc < ns ? bx + r0 + rc : ns;
+    const int buf = 2 * bt * (bx + rc), ui = (bt + tc) * m.ucols;
     m.ut = buf > ui ? buf : ui;
-    m.s = m.ut + (bt + kLoopChunk - 1) * m.ucols;
-    m.total = m.s + kTopPitch * (bt + kLoopChunk) * bx;
+    m.s = m.ut + (bt + tc - 1) * m.ucols;
+    m.total = m.s + top_pitch(rc) * (bt + tc) * bx;
     return m;
 }
 
@@ -83,7 +88,9 @@ __host__ __device__ constexpr TileSmem tile_smem(int bx, int bt, int ns, int r0)
 // chunk of R.  (Narrower tiles have more rows, but at most 256 sites all the
 // same, and their staged rows end at the extent.)
 constexpr size_t kTileMaxSmem =
-    sizeof(float4) * (size_t)tile_smem(kTileMaxBx, kTileThreads / kTileMaxBx, 1 << 20, kWilsonMaxR - kLoopChunk).total;
+    sizeof(float4) * (size_t)tile_smem(kTileMaxBx, kTileThreads / kTileMaxBx, kLoopChunk, kLoopChunk, 1 << 20,
+                                       kWilsonMaxR - kLoopChunk)
+                         .total;
 
 // FULL: the chunk has all eight R (no test per R in the inner loop).
 template <bool FULL>
@@ -95,7 +102,8 @@ __global__ void __launch_bounds__(kTileThreads, 3)
     // [T][R][h, l] of the chunk, modulo 2^32; starts at minus what the bits of
     // 6 add up to over the block's warps
     __shared__ unsigned int s_sum[2 * kLoopChunk * kLoopChunk];
-    const int pitch = tl.bx + kLoopChunk;  // a T_T row: the tile's columns, then x + R
+    const int rc = FULL ? kLoopChunk : tl.rc, tp = top_pitch(rc);
+    const int pitch = tl.bx + rc;  // a T_T row: the tile's columns, then x + R
     const int buf_len = tl.bt * pitch;
     uint32_t b = blockIdx.x;
     const int r0 = (int)(b % (uint32_t)tl.nr) * kLoopChunk;
@@ -113,7 +121,7 @@ __global__ void __launch_bounds__(kTileThreads, 3)
     const int t0 = (int)(b % (uint32_t)tl.nt) * tl.bt;
     const int i = (int)(b / (uint32_t)tl.nt);
     const int rcnt = FULL ? kLoopChunk : min(kLoopChunk, rmax - r0), tcnt = min(kLoopChunk, tmax - tc0);
-    const TileSmem lay = tile_smem(tl.bx, tl.bt, g.ns, r0);
+    const TileSmem lay = tile_smem(tl.bx, tl.bt, rc, tl.tc, g.ns, r0);
     float4 *const s_ui = sm, *const s_ut = sm + lay.ut;
     float4 *const s_buf = sm + lay.s;  // [row t0 + tc0 + j][column][R]
     const int stride_i = g.stride[i];
@@ -140,7 +148,7 @@ __global__ void __launch_bounds__(kTileThreads, 3)
     for (int q = threadIdx.x; q < (tl.bt + tcnt) * tl.bx; q += blockDim.x) {
         const int j = q / tl.bx;
         const float4 *const u = s_ui + j * lay.ucols;
-        float4 *const to = s_buf + q * kTopPitch;
+        float4 *const to = s_buf + q * tp;
         int d = q - j * tl.bx;
         float4 s = u[d];
         if (r0 == 0) to[0] = s;
@@ -166,7 +174,7 @@ __global__ void __launch_bounds__(kTileThreads, 3)
     __syncthreads();  // s_buf is complete, the staged U_i is done with
     if (tc0 == 0) {
 #pragma unroll
-        for (int r = 0; r < kLoopChunk; ++r) s_bot[r] = s_buf[site * kTopPitch + min(r, rcnt - 1)];
+        for (int r = 0; r < kLoopChunk; ++r) s_bot[r] = s_buf[site * tp + min(r, rcnt - 1)];
     } else {  // the site's own row is not among the staged ones
         int a = (x0 + c) % g.ns;
         const int t = (t0 + k) % g.nt;
@@ -204,7 +212,7 @@ __global__ void __launch_bounds__(kTileThreads, 3)
     const int tb_off = wrap_once(c + r0, lay.ucols) - c;
     const float4 *ut_h = s_ut + hk * lay.ucols + wrap_once(tl.bx + r0 + h, lay.ucols);
     float4 *own_to = sm + k * pitch + c, *halo_to = sm + hk * pitch + tl.bx + h;
-    const float4 *top = s_buf + (site + tl.bx) * kTopPitch;  // the site one step of T above, then two ...
+    const float4 *top = s_buf + (site + tl.bx) * tp;  // the site one step of T above, then two ...
 
     const int lane = threadIdx.x & 31;
     bool outside = false;
@@ -254,7 +262,7 @@ __global__ void __launch_bounds__(kTileThreads, 3)
                 }
             }
         }
-        top += tl.bx * kTopPitch;
+        top += tl.bx * tp;
         if ((tt & 3) == 3) flush(tt - 3);
     }
     if (tcnt & 3) flush(tcnt & ~3);
@@ -297,8 +305,9 @@ __global__ void wilson_tile_finish_kernel(const unsigned long long *__restrict__
 // One launch per T: each thread takes (site, direction) items and, for R = 1
 // .. rmax, extends S_R and the line at height T by one link and walks
 // T_T(x+Ri); per-R binary64 sums in registers, block partials in a fixed
-// order.  Takes any links, so it finishes the calls whose loops the tiled
-// kernel's fixed point does not hold (24^4 up to 8 x 8: 1.2 ms).
+// order.  The faster one for few small loops (walks_are_faster), and as it takes
+// any links it finishes the calls whose loops the tiled kernel's fixed point
+// does not hold (24^4 up to 8 x 8: 1.2 ms).
 struct Site {
     int c[4];
 };
@@ -390,66 +399,99 @@ __global__ void wilson_finish_kernel(const double *__restrict__ partials, int nb
     }
 }
 
+// Enqueues the walks; the values go to the reduction scratch, behind the
+// block partials.  *d_out: their device address.
 template <int RM>
-static cudaError_t launch_wilson(su2_lattice *lat, int rmax, int tmax, double *d_out)
+static cudaError_t launch_wilson(su2_lattice *lat, int rmax, int tmax, double **d_out)
 {
     const Geom g = geom_of(lat);
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, lat->device);
-    const int grid = grid_for(6 * (int64_t)g.vh, kWilsonThreads, std::min(4 * sms, lat->scratch.partials_cap / rmax));
+    const int room = (lat->scratch.partials_cap - rmax * tmax) / rmax;
+    const int grid = grid_for(6 * (int64_t)g.vh, kWilsonThreads, std::min(4 * sms, room));
     const double scale = 1.0 / (6.0 * (double)g.vh);
+    *d_out = lat->scratch.partials + (size_t)grid * rmax;
     for (int T = 1; T <= tmax; ++T) {
         wilson_kernel<RM><<<grid, kWilsonThreads, 0, lat->stream>>>(lat->links, g, rmax, T, lat->scratch.partials);
         wilson_finish_kernel<<<1, kWilsonThreads, 0, lat->stream>>>(lat->scratch.partials, grid, rmax, T, tmax,
-                                                                   scale, d_out);
+                                                                   scale, *d_out);
     }
     return cudaGetLastError();
 }
 
-// Enqueues the tiled kernel: tiles of whole rows (up to 64 columns) and as
-// many time slices as fit 256 threads.  The sums live in the reduction
-// scratch, in as many slots as fit (blocks spread over the slots, so their
-// atomics meet rarely), the results behind them: rmax tmax values and the
-// flag.  *d_out: their device address.
+static cudaError_t launch_walks(su2_lattice *lat, int rmax, int tmax, double **d_out)
+{
+    return rmax <= 4   ? launch_wilson<4>(lat, rmax, tmax, d_out)
+           : rmax <= 8 ? launch_wilson<8>(lat, rmax, tmax, d_out)
+                       : launch_wilson<16>(lat, rmax, tmax, d_out);
+}
+
+// The tiles of a call: whole rows (more than 64 columns in even parts) and as
+// many time slices as fit 256 threads, in even tiles.
+static LoopTiles loop_tiles(int ns, int nt, int rmax, int tmax)
+{
+    LoopTiles tl;
+    tl.nx = (ns + kTileMaxBx - 1) / kTileMaxBx;
+    tl.bx = (ns + tl.nx - 1) / tl.nx;
+    tl.bt = std::min(nt, std::max(1, kTileThreads / tl.bx));
+    tl.nt = (nt + tl.bt - 1) / tl.bt;
+    tl.bt = (nt + tl.nt - 1) / tl.nt;
+    tl.rc = std::min(rmax, kLoopChunk);
+    tl.tc = std::min(tmax, kLoopChunk);
+    tl.nr = (rmax + kLoopChunk - 1) / kLoopChunk;
+    tl.ntc = (tmax + kLoopChunk - 1) / kLoopChunk;
+    return tl;
+}
+
+static int tile_threads(const LoopTiles &tl) { return std::max(32, (tl.bx * tl.bt + 31) & ~31); }
+
+// The walks load, per site and direction, T links of the line at the site and
+// for each R one of S_R, one of its top and T of the far line: `loads` for all
+// extents, at about 3 ps each (48^4) and 13 us per launch (one per T).  A tile
+// costs 14 to 15 such loads per chunk before its first loop, over the threads
+// that its sites leave idle (more on a large lattice, less on one that stays
+// in L2), and little per loop after it.  So the walks stay the faster ones for
+// few small loops, from about 20^4 on (16^4, 3 x 1: 41 / 36).  us per call on
+// the walks / the tiles:
+//   R x T        1 x 1       2 x 1       4 x 1       2 x 2       4 x 2       8 x 1
+//   24^4       43 / 68     54 / 69     68 / 72     94 / 74    132 / 85    116 / 82
+//   48^4     217 / 728   352 / 790   658 / 900   753 / 936 1417 / 1099  1325 / 947
+static bool walks_are_faster(const su2_lattice *lat, int rmax, int tmax)
+{
+    const LoopTiles tl = loop_tiles(lat->ns, lat->nt, rmax, tmax);
+    const double vol = (double)lat->vol, chunks = tl.nr * tl.ntc;
+    const double loads = 0.5 * tmax * (tmax + 1) * (1 + rmax) + 2.0 * tmax * rmax;
+    const double filled = (double)lat->ns * lat->nt / ((double)tl.nx * tl.nt * tile_threads(tl));
+    const double most = vol < 1e6 ? 14.0 : chunks == 1.0 ? 22.0 : 18.0 * chunks;
+    return loads * filled <= most && vol >= 1e5 + 3e5 * (tmax - 1);
+}
+
+// Enqueues the tiled kernel.  The sums live in the reduction scratch, in as many slots as fit (blocks spread over
+// the slots, so their atomics meet rarely), the results behind them: rmax tmax
+// values and the flag.  *d_out: their device address.
 static cudaError_t launch_tiles(su2_lattice *lat, int rmax, int tmax, double **d_out)
 {
     const Geom g = geom_of(lat);
     const int n_out = rmax * tmax;
-    LoopTiles tl;
-    tl.bx = std::min(g.ns, kTileMaxBx);
-    tl.bt = std::min(lat->nt, std::max(1, kTileThreads / tl.bx));
-    tl.nx = (g.ns + tl.bx - 1) / tl.bx;
-    tl.nt = (lat->nt + tl.bt - 1) / tl.bt;
-    tl.bt = (lat->nt + tl.nt - 1) / tl.nt;  // even tiles
-    tl.nr = (rmax + kLoopChunk - 1) / kLoopChunk;
-    tl.ntc = (tmax + kLoopChunk - 1) / kLoopChunk;
+    const LoopTiles tl = loop_tiles(g.ns, lat->nt, rmax, tmax);
     const int nslots = std::min(256, (lat->scratch.partials_cap - n_out - 2) / (2 * n_out));
     unsigned long long *slots = (unsigned long long *)lat->scratch.partials;
     unsigned int *flag = (unsigned int *)(slots + (size_t)nslots * 2 * n_out);
     *d_out = (double *)(flag + 2);
     cudaError_t e = cudaMemsetAsync(slots, 0, sizeof(double) * ((size_t)nslots * 2 * n_out + 1), lat->stream);
     if (e != cudaSuccess) return e;
-    const size_t smem = sizeof(float4) * (size_t)tile_smem(tl.bx, tl.bt, g.ns, (tl.nr - 1) * kLoopChunk).total;
+    const size_t smem = sizeof(float4) * (size_t)tile_smem(tl.bx, tl.bt, tl.rc, tl.tc, g.ns, (tl.nr - 1) * kLoopChunk).total;
     const auto kernel = rmax % kLoopChunk == 0 ? wilson_tile_kernel<true> : wilson_tile_kernel<false>;
     // the limit belongs to the kernel, which other threads launch too: always the most that a tile takes
     e = smem <= kTileMaxSmem ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileMaxSmem)
                              : cudaErrorInvalidValue;
     if (e != cudaSuccess) return e;
     const unsigned int blocks = 3u * (unsigned int)(g.ns * g.ns) * (unsigned int)(tl.nx * tl.nt * tl.nr * tl.ntc);
-    const int threads = std::max(32, (tl.bx * tl.bt + 31) & ~31);
-    kernel<<<blocks, threads, smem, lat->stream>>>(lat->links, g, tl, rmax, tmax, slots, nslots, flag);
+    kernel<<<blocks, tile_threads(tl), smem, lat->stream>>>(lat->links, g, tl, rmax, tmax, slots, nslots, flag);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     wilson_tile_finish_kernel<<<n_out, 32, 0, lat->stream>>>(slots, nslots, n_out, 1.0 / (6.0 * (double)g.vh), flag,
                                                              *d_out);
     return cudaGetLastError();
-}
-
-// The binary64 path: d_out holds rmax tmax values.
-static cudaError_t launch_walks(su2_lattice *lat, int rmax, int tmax, double *d_out)
-{
-    return rmax <= 4   ? launch_wilson<4>(lat, rmax, tmax, d_out)
-           : rmax <= 8 ? launch_wilson<8>(lat, rmax, tmax, d_out)
-                       : launch_wilson<16>(lat, rmax, tmax, d_out);
 }
 
 }  // namespace su2
@@ -465,29 +507,20 @@ extern "C" su2_status su2_wilson_loops(su2_lattice *lat, int rmax, int tmax, dou
     }
     DeviceGuard guard(lat->device);
     const size_t n_out = (size_t)rmax * (size_t)tmax;
-    const size_t bytes = sizeof(double) * n_out;
     HostPage page(lat->stream);
     double own[kWilsonMaxR * kWilsonMaxT + 1];
     double *const host = page.p ? (double *)page.p : own;
-    double *d_tiles = nullptr;
-    SU2_CUDA(launch_tiles(lat, rmax, tmax, &d_tiles));
-    SU2_CUDA(cudaMemcpyAsync(host, d_tiles, bytes + sizeof(double), cudaMemcpyDeviceToHost, lat->stream));
-    SU2_CUDA(cudaStreamSynchronize(lat->stream));
+    double *d_out = nullptr;
+    bool walk = walks_are_faster(lat, rmax, tmax);
+    for (;;) {
+        SU2_CUDA(walk ? launch_walks(lat, rmax, tmax, &d_out) : launch_tiles(lat, rmax, tmax, &d_out));
+        const size_t n = walk ? n_out : n_out + 1;  // the tiles' values are followed by their flag
+        SU2_CUDA(cudaMemcpyAsync(host, d_out, sizeof(double) * n, cudaMemcpyDeviceToHost, lat->stream));
+        SU2_CUDA(cudaStreamSynchronize(lat->stream));
+        if (walk || host[n_out] == 0.0) break;
+        walk = true;  // a loop outside (-2, 2)
+    }
     page.settled();
-    if (host[n_out] == 0.0) {
-        std::copy(host, host + n_out, out);
-        return SU2_OK;
-    }
-    // a loop outside (-2, 2)
-    double *d_out = (double *)device_alloc(bytes, lat->device, lat->stream);
-    if (!d_out) {
-        set_last_error("device allocation for the Wilson loops failed");
-        return SU2_E_NOMEM;
-    }
-    cudaError_t e = launch_walks(lat, rmax, tmax, d_out);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out, d_out, bytes, cudaMemcpyDeviceToHost, lat->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(lat->stream);
-    device_free(d_out, bytes, lat->device, lat->stream);
-    SU2_CUDA(e);
+    std::copy(host, host + n_out, out);
     return SU2_OK;
 }
