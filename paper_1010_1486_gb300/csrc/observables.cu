@@ -9,6 +9,7 @@
 #include <algorithm>
 
 #include "observables.cuh"
+#include "plaquette_plan.h"
 #include "su2_device.cuh"
 #include "su2_internal.h"
 
@@ -23,26 +24,27 @@ namespace su2 {
 // One site per thread in lexicographic order (sixteen loads, two runs of 256
 // bytes each) was bound by L1 wavefronts (88%), and the same by even/odd order
 // by the traffic from L2 (87 us, 12.7 TB/s).  48^4: 100 -> 90 us per call, 82 us
-// (ncu) in the kernel, which waits for its loads (24 warps per SM, 78
+// (ncu) in the kernel, which waits for its loads (24 warps per SM, 80
 // registers); splitting the planes into two groups of loads, one in flight
 // while the other is computed, spills (102 us) or halves the warps (106 us).
-constexpr int kPlaqPairs = 384;                 // pairs of sites (2 j, 2 j + 1) per block
 constexpr int kPlaqThreads = 2 * kPlaqPairs;    // one block per SM
 
 // dst (+ *idx when idx is given: the measurement slot of a graph replay)
-__global__ void __launch_bounds__(kPlaqThreads, 1) plaquette_kernel(const float4 *__restrict__ L, Geom g, int pair_blocks,
-                                                                  int t_chunk, double *__restrict__ partials,
+__global__ void __launch_bounds__(kPlaqThreads, 1) plaquette_kernel(const float4 *__restrict__ L, Geom g, PlaquettePlan pl,
+                                                                  double *__restrict__ partials,
                                                                   unsigned int *__restrict__ ticket,
                                                                   double *__restrict__ dst,
                                                                   const uint32_t *__restrict__ idx)
 {
     double acc = 0.0;
     const int half = g.vs >> 1;
-    const int chunk = (int)blockIdx.x / pair_blocks;
     const int sp = (int)threadIdx.x >= kPlaqPairs;  // spatial parity, warp-uniform
-    const int j = ((int)blockIdx.x - chunk * pair_blocks) * kPlaqPairs + (int)threadIdx.x - sp * kPlaqPairs;
-    const int t0 = chunk * t_chunk, t1 = min(t0 + t_chunk, g.nt);
-    if (j < half && t0 < t1) {
+#pragma unroll 1
+    for (int item = (int)blockIdx.x; item < pl.items; item += (int)gridDim.x) {
+        const int chunk = item / pl.pair_blocks;
+        const int j = (item - chunk * pl.pair_blocks) * kPlaqPairs + (int)threadIdx.x - sp * kPlaqPairs;
+        const int t0 = chunk * pl.t_chunk, t1 = min(t0 + pl.t_chunk, g.nt);
+        if (j >= half) continue;
         const uint32_t r1 = fastdiv(2u * (uint32_t)j, g.div_ns), z = fastdiv(r1, g.div_ns);
         const int y = (int)(r1 - z * (uint32_t)g.ns);
         const int x = 2 * j - (int)r1 * g.ns + ((y + (int)z + sp) & 1);
@@ -207,14 +209,10 @@ su2_status launch_plaquette(su2_lattice *lat, double *dst)
     const Geom g = geom_of(lat);
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, lat->device);
-    // one block per SM: the time extent in as many chunks as fill them
-    const int pair_blocks = (g.vs / 2 + kPlaqPairs - 1) / kPlaqPairs;
-    const int chunks = std::max(1, std::min(lat->nt, sms / pair_blocks));
-    const int t_chunk = (lat->nt + chunks - 1) / chunks;
-    const int grid = pair_blocks * ((lat->nt + t_chunk - 1) / t_chunk);
-    plaquette_kernel<<<grid, kPlaqThreads, 0, lat->stream>>>(lat->links, g, pair_blocks, t_chunk,
-                                                             lat->scratch.partials, lat->scratch.ticket, dst,
-                                                             lat->capturing ? lat->d_ctr + 1 : nullptr);
+    const PlaquettePlan pl = plaquette_plan(g.vs, lat->nt, sms);
+    plaquette_kernel<<<pl.grid, kPlaqThreads, 0, lat->stream>>>(lat->links, g, pl, lat->scratch.partials,
+                                                                lat->scratch.ticket, dst,
+                                                                lat->capturing ? lat->d_ctr + 1 : nullptr);
     SU2_CUDA(cudaGetLastError());
     return SU2_OK;
 }
