@@ -568,8 +568,12 @@ __global__ void adam_kernel(float *w, float *m, float *v, const float *partials,
 // w[1946]: block sums in binary64, added in block order by the block that
 // finishes last (the ticket returns to 0).  One block for all pairs waited
 // for its loads 780 times over 200,000 pairs (255 us under ncu); with a block
-// per 2048 pairs, up to one per SM, 13 us.
+// per 2048 pairs, up to one per SM, 13 us.  Up to kScalingOneBlock pairs one
+// block is as fast or faster, as it needs no ticket: us per call, one block for
+// all pairs / the ticket always / this, 2 pairs 13.0 / 15.4 / 13.1, 2048 15.2 / 18.1 / 15.4,
+// 4096 18.0 / 18.0 / 18.0, 10,000 25.5 / 18.6 / 18.3.
 constexpr int kScalingThreads = 256;
+constexpr size_t kScalingOneBlock = 4096;
 
 __global__ void __launch_bounds__(kScalingThreads)
     input_scaling_kernel(const float2 *__restrict__ pairs, long long n, double *__restrict__ sums,
@@ -582,31 +586,31 @@ __global__ void __launch_bounds__(kScalingThreads)
         a += x;
         b += x * x;
     }
-    a = block_sum(a);
-    b = block_sum(b);
-    __shared__ bool last;
-    if (threadIdx.x == 0) {
-        sums[2 * blockIdx.x] = a;
-        sums[2 * blockIdx.x + 1] = b;
+    block_sum2(a, b);
+    if (gridDim.x > 1) {
+        __shared__ bool last;
+        if (threadIdx.x == 0) {
+            sums[2 * blockIdx.x] = a;
+            sums[2 * blockIdx.x + 1] = b;
+            __threadfence();
+            last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        }
+        __syncthreads();
+        if (!last) return;
         __threadfence();
-        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        a = b = 0.0;
+        for (unsigned int i = threadIdx.x; i < gridDim.x; i += blockDim.x) {
+            a += ((volatile double *)sums)[2 * i];
+            b += ((volatile double *)sums)[2 * i + 1];
+        }
+        block_sum2(a, b);
+        if (threadIdx.x == 0) *ticket = 0u;
     }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    a = b = 0.0;
-    for (unsigned int i = threadIdx.x; i < gridDim.x; i += blockDim.x) {
-        a += ((volatile double *)sums)[2 * i];
-        b += ((volatile double *)sums)[2 * i + 1];
-    }
-    a = block_sum(a);
-    b = block_sum(b);
     if (threadIdx.x == 0) {
         const double mean = a / (double)n;
         const double var = b / (double)n - mean * mean;
         w[learned::kOffMean] = (float)mean;
         w[learned::kOffScale] = (float)(1.0 / sqrt(var > 1e-12 ? var : 1e-12));
-        *ticket = 0u;
     }
 }
 
@@ -772,7 +776,8 @@ su2_status su2_trainer_set_input_scaling(su2_trainer *tr, const float *dev_pairs
     if (!tr || !dev_pairs || n < 2) return SU2_E_INVAL;
     DeviceGuard guard(tr->device);
     // the block sums take the head of the step partials, idle between calls
-    const int grid = (int)std::min<size_t>((n + 2047) / 2048, (size_t)tr->sms);
+    const int grid =
+        n <= train::kScalingOneBlock ? 1 : (int)std::min<size_t>((n + 2047) / 2048, (size_t)tr->sms);
     train::input_scaling_kernel<<<grid, train::kScalingThreads, 0, tr->stream>>>(
         (const float2 *)dev_pairs, (long long)n, (double *)tr->partials, tr->err + 16, tr->w);
     SU2_CUDA(cudaGetLastError());

@@ -32,3 +32,21 @@ def test_overlapped_steps_equal_separate_ones(batch, steps):
     assert np.array_equal(la.view(np.uint32), lb.view(np.uint32))
     assert np.array_equal(wa.view(np.uint32), wb.view(np.uint32))
     assert np.isfinite(la).all() and la[-5:].mean() < la[:5].mean()
+
+
+@pytest.mark.parametrize("n", [4095, 4096, 4097, 6145])
+def test_input_scaling_either_side_of_one_block(n):
+    torch = pytest.importorskip("torch")
+    x = np.random.default_rng(n).normal(12.0, 3.0, n).astype(np.float32)
+    dev = torch.from_numpy(np.stack([x, np.zeros_like(x)], axis=1)).cuda()
+    tr = su2.su2_trainer_create(learn.initial_weights(5), 9)
+    try:
+        for _ in range(2):  # the second call finds the ticket re-armed
+            su2.su2_trainer_set_input_scaling(tr, dev.data_ptr(), n)
+            w = su2.su2_trainer_get_weights(tr)
+            # one rounding to binary32 of each value, binary64 sums before it
+            x64 = x.astype(np.float64)
+            assert abs(w[1945] - x64.mean()) <= 2.0 ** -23 * abs(x64.mean())
+            assert abs(w[1946] * x64.std() - 1.0) <= 2.0 ** -22
+    finally:
+        su2.su2_trainer_destroy(tr)
