@@ -73,7 +73,7 @@ typedef struct {
     uint64_t link_updates;      /* 4 V per sweep                                              */
     uint64_t trials[8];         /* heat-bath a0 trials of phase 2*mu + parity, summed over sweeps */
     uint64_t sampler_failures;  /* links whose draw hit the trial cap                         */
-    uint32_t kernel_launches;   /* heat-bath phase launches (8 per sweep)                     */
+    uint32_t kernel_launches;   /* heat-bath phases run, 8 per sweep: a launch each, but for small lattices (su2_generate) */
     uint32_t timed;             /* 1 if kernel_ms / overrelax_ms are valid (su2_set_timing)   */
     double kernel_ms;           /* summed device time of the heat-bath phase kernels          */
     uint64_t overrelax_sweeps;  /* over-relaxation sweeps performed (see su2_set_overrelax)   */
@@ -127,7 +127,9 @@ su2_status su2_heatbath_phase(su2_lattice *lat, int mu, int parity);
  * staple terms S of the directions nu < mu); it equals su2_plaquette on the
  * same links up to binary32 rounding of the single plaquettes.  A sweep
  * reunitarized before its measurement uses the separate plaquette pass.
- * On a lattice created with a stream (not the legacy default stream) and
+ * With timing off, a lattice of at most 8,192 links per phase (V <= 16,384)
+ * takes up to 256 sweeps, their measurements included, in one launch.  On a
+ * larger lattice created with a stream (not the legacy default stream) and
  * with timing off, each sweep is replayed from a CUDA graph captured on first
  * use (the sweep counter and the measurement slot are kept on the device;
  * the graph is captured again when the sampler, beta, seed, over-relaxation,
