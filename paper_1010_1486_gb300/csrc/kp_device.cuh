@@ -45,9 +45,11 @@ __device__ __forceinline__ bool kp_candidate(float num, uint32_t w3, float two_b
     return lam2 <= 1.0f && __fmul_rn(r4, r4) <= __fsub_rn(1.0f, lam2);
 }
 
-// One trial (block t of the KP stream).  IN_RANGE: 2 beta k is within the
-// range of div_in_range (the numerator is 0 or above 2^-80: |ln| >= 2^-24
-// unless zero, cos^2 >= 2^-43).
+// One trial (block t of the KP stream).  IN_RANGE: 2 beta k is at most 2^61.
+// The numerator is 0 or above 2^-67 (|ln| >= 2^-24 unless zero, cos^2 >= 2^-43),
+// so from beta k = 2^22 on the quotient can fall below the range in which
+// div_in_range is correctly rounded.  Both forms are then below 2^-89, and the
+// trial takes only 1 - 2 l and 1 - l of it, which are 1.
 template <bool IN_RANGE = false, bool CHECKED_LOG = false>
 __device__ __forceinline__ bool kp_trial(uint4 w, float two_bk, float &a0)
 {
