@@ -71,7 +71,10 @@ constexpr int kRetryCap = 64;  // per warp: at most 31 left over + 32 pushed by 
 // results, so the main path has no divergent branch.  MEAS: the plaquette
 // contributions (1/2) Tr U'S, S the staple terms of nu < MU, as in the
 // Creutz kernel.
-template <int MU, bool MEAS, bool SLAB>
+//
+// PEEL: a warp's last round runs without loads of a next one, as in the heat-bath
+// kernel (peel_kp: where that pays).
+template <int MU, bool MEAS, bool SLAB, bool PEEL>
 __global__ void __launch_bounds__(kKpThreads, kKpMinBlocks) kp_phase_kernel(const KpParams p)
 {
     // a time slab: interior eo range, random numbers of the global site
@@ -251,9 +254,13 @@ __global__ void __launch_bounds__(kKpThreads, kKpMinBlocks) kp_phase_kernel(cons
         sp_cur = sp_next;
         even_round = !even_round;
     };
-    if (base < eo_end) {  // warp-uniform
-        while (base + stride < eo_end) round(std::true_type{});
-        round(std::false_type{});
+    if (PEEL) {
+        if (base < eo_end) {  // warp-uniform
+            while (base + stride < eo_end) round(std::true_type{});
+            round(std::false_type{});
+        }
+    } else {
+        while (base < eo_end) round(std::true_type{});
     }
     if (queued > 0) retry(0, queued);
     const unsigned int wsum = __reduce_add_sync(0xffffffffu, trials);
@@ -267,7 +274,21 @@ __global__ void __launch_bounds__(kKpThreads, kKpMinBlocks) kp_phase_kernel(cons
     }
 }
 
-template <int MU, bool MEAS, bool SLAB = false>
+// Whether the last round is peeled.  The retry pass is then in the code three
+// times instead of twice.  Where it holds a mixture of many links with beta k <
+// 2 (Creutz's method, a long pass) and of rejected ones, in many rounds, that
+// costs more than the peeled round gives, from a number of rounds on that grows
+// with beta.  us per phase with / without at 32^4 (4.5 rounds), 40^4 (11) and
+// 48^4 (22.7): beta = 0.3 28.8 / 30.0, 64.3 / 65.6, 128 / 130; 0.5 38.0 / 33.1,
+// 81.1 / 72.1, 147 / 141; 1.0 31.7 / 29.4, 70.3 / 62.1, 128 / 118; 1.5 21.9 /
+// 23.1, 51.8 / 49.2, 90.3 / 87.9; 2.3 18.9 / 20.8, 40.8 / 41.3, 75.8 / 75.9.
+static bool peel_kp(float beta, float rounds)
+{
+    const float over = beta > 1.0f ? beta - 1.0f : 0.0f;
+    return !(beta >= 0.45f && beta < 2.25f && rounds > 3.7f + 11.0f * over * over);
+}
+
+template <int MU, bool MEAS, bool SLAB = false, bool PEEL = true>
 static cudaError_t launch_kp(const KpParams &p, su2_lattice *lat)
 {
     static int per_sm[64] = {};
@@ -276,7 +297,7 @@ static cudaError_t launch_kp(const KpParams &p, su2_lattice *lat)
     if (device < 0 || device >= 64) device = 0;
     if (!per_sm[device]) {
         cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[device],
-                                                                      kp_phase_kernel<MU, MEAS, SLAB>, kKpThreads, 0);
+                                                                      kp_phase_kernel<MU, MEAS, SLAB, PEEL>, kKpThreads, 0);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms[device], cudaDevAttrMultiProcessorCount, device);
         if (e != cudaSuccess) return e;
         per_sm[device] = std::max(1, per_sm[device]);
@@ -284,8 +305,10 @@ static cudaError_t launch_kp(const KpParams &p, su2_lattice *lat)
     const int n = SLAB ? p.slab.eo_end - p.slab.eo_begin : p.g.vh;
     const int want = (n + kKpThreads - 1) / kKpThreads;
     const int grid = std::max(1, std::min(std::min(want, per_sm[device] * sms[device]), kFusedSlots));
+    if (PEEL && !peel_kp(p.beta, (float)n / (float)(grid * kKpThreads)))
+        return launch_kp<MU, MEAS, SLAB, false>(p, lat);
     if (MEAS) fused_launched(lat, MU, 0, grid);
-    kp_phase_kernel<MU, MEAS, SLAB><<<grid, kKpThreads, 0, lat->stream>>>(p);
+    kp_phase_kernel<MU, MEAS, SLAB, PEEL><<<grid, kKpThreads, 0, lat->stream>>>(p);
     return cudaGetLastError();
 }
 
