@@ -81,10 +81,10 @@ constexpr int kCrMinBlocks = SU2_HB_MIN_BLOCKS;  // blocks per SM the register b
 // trip to memory at the end of every launch; but the loop body is then in the
 // code twice, and at many rounds per warp the compiler's schedule of the pair
 // is the slower one.  us per phase with and without, measured every sweep,
-// beta = 4: 20^4 14.3 / 15.7, 24^4 17.9 / 19.4, 32^4 30.8 / 32.0, 36^4 (7.2
-// rounds) 44.8 / 45.5, 40^4 (11) 61.3 / 61.5, 44^4 83.8 / 83.2, 48^4 (22.7)
-// 113.6 / 111.8 (all with separate queues; one array has since taken 1 us off
-// both at 24^4 and 3 at 48^4); so up to kCrPeelRounds.
+// beta = 4: 20^4 13.9 / 15.4, 24^4 17.6 / 19.1, 32^4 30.2 / 31.8, 36^4 (7.2
+// rounds) 43.8 / 44.9, 40^4 (11) 59.8 / 60.7, 44^4 (16) 81.1 / 81.7, 48^4 (22.7)
+// 110.1 / 109.8; without measurement 40^4 58.2 / 58.2, 44^4 78.8 / 78.7, 48^4
+// 106.5 / 105.3; so up to kCrPeelRounds.
 constexpr int kCrPeelRounds = 10;
 
 template <int MU, bool MEAS, bool SLAB, bool PEEL>

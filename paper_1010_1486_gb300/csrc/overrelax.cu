@@ -40,9 +40,9 @@ struct OrParams {
 // heat-bath kernels.
 //
 // PEEL: a warp's last round runs without loads of a next one, as in the
-// heat-bath kernel.  us per phase with and without, beta = 4: 20^4 5.1 / 6.2,
-// 24^4 6.2 / 8.2, 28^4 8.2 / 10.2, 32^4 (3.4 rounds) 12.0 / 12.3, 36^4 (5.4)
-// 22.8 / 22.9, 40^4 (8.2) 32.4 / 31.6, 48^4 (17) 62.2 / 61.0; so up to
+// heat-bath kernel.  us per phase with and without, beta = 4: 20^4 5.4 / 6.4,
+// 24^4 6.4 / 8.5, 28^4 8.6 / 10.5, 32^4 (3.4 rounds) 12.6 / 13.0, 36^4 (5.4)
+// 23.4 / 23.3, 40^4 (8.2) 33.1 / 32.3, 48^4 (17) 62.7 / 61.6; so up to
 // kOrPeelRounds.
 constexpr int kOrPeelRounds = 6;
 
