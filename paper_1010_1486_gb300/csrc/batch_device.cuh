@@ -74,9 +74,9 @@ __device__ __forceinline__ unsigned long long global_time_ns()
 }
 
 // Grid-wide barrier number `passed` (0, 1, ...) of a cooperative launch (all
-// blocks co-resident; `blocks` of them arrive at each barrier).  Arrival is one release-acquire atomic per block, and
-// the waits poll with acquire loads; the clock is read every kBarrierPolls
-// polls only.  Every wait is bounded by timeout_ns: on expiry the block sets
+// blocks co-resident; `blocks` of them arrive at each barrier).  Arrival is one
+// release-acquire atomic per block, and the waits poll with acquire loads; the
+// clock is read every kBarrierPolls polls only.  Every wait is bounded by timeout_ns: on expiry the block sets
 // bar->error and releases the others; the function then returns false
 // everywhere and the caller abandons the sweep.  (With both numbers on one
 // line, a clock read and 100 ns of sleep per poll, and all co-resident blocks
@@ -409,9 +409,10 @@ __global__ void __launch_bounds__(T, kBatchThreadsPerSm / T) batch_sweep_kernel(
     const int wib = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int warp_global = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (*(volatile unsigned int *)&bp.bar->error & 1u) return;  // an earlier launch of the call was given up
+    const unsigned int error = *(volatile unsigned int *)&bp.bar->error;
     const uint32_t sweep = *(volatile unsigned int *)bp.sweep;
     const unsigned int slot = *(volatile unsigned int *)bp.meas_index;
+    if (error & 1u) return;  // an earlier launch of the call was given up
     const bool fused = bp.fused && (int)slot < bp.history_cap;
     bool ok = true;
     unsigned int barriers = 0;
